@@ -7,20 +7,15 @@
 // vectors (BF16).  The output is written with streaming stores so that it
 // does not evict the table from L2.
 //
-// The backward uses red.global.add.v4.f32 (one 16-byte vector reduction per
-// corner and level), accumulating into an FP32 gradient table.
+// The backward reduces 16-byte rows into an FP32 gradient table
+// (red.global.add.v4.f32), after merging the coarse levels' contributions of
+// consecutive points (adjoint_impl.cuh).
 #include <algorithm>
 
-#include "hashgrid_impl.cuh"
+#include "adjoint_impl.cuh"
 
 namespace inpc {
 namespace {
-
-// The adjoint processes levels in groups of kLevelGroup along grid y: blocks are
-// dispatched in linear order, so all points visit one group of levels
-// before the next, and the rows touched at a time (one or two 8 MB levels)
-// stay resident in L2 instead of the whole table.
-constexpr int kLevelGroup = 2;
 
 // A warp takes 16 consecutive points, two lanes per point, through the
 // levels of one level group (grid y, plan_level_groups), two levels at a
@@ -74,41 +69,78 @@ __global__ void __launch_bounds__(256) k_hash_fwd(GridParams P, LevelGroups LG, 
 }
 
 
-__global__ void __launch_bounds__(256) k_hash_bwd(GridParams P, const float* __restrict__ pos,
-                                                  const float* __restrict__ dh, long long n,
-                                                  float* __restrict__ grad) {
-  const int l0 = blockIdx.y * kLevelGroup;
-  const int gl = min(kLevelGroup, P.n_levels - l0);
-  const long long total = n * gl;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const long long p = i / gl;
-    const int l = l0 + (int)(i - p * gl);
-    const float4 g = __ldcs(reinterpret_cast<const float4*>(dh) + p * P.n_levels + l);
-    if (g.x == 0.f && g.y == 0.f && g.z == 0.f && g.w == 0.f) continue;
-    uint32_t cx, cy, cz;
-    float gx[2], gy[2], gz[2];
-    const int N = P.res[l];
-    cell_frac(__ldg(pos + 3 * p + 0), N, cx, gx[0], gx[1]);
-    cell_frac(__ldg(pos + 3 * p + 1), N, cy, gy[0], gy[1]);
-    cell_frac(__ldg(pos + 3 * p + 2), N, cz, gz[0], gz[1]);
-    float* gl_ = grad + 4 * P.offset[l];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int bx = c & 1, by = (c >> 1) & 1, bz = (c >> 2) & 1;
-      const float w = gx[bx] * gy[by] * gz[bz];
-      const uint32_t row = vertex_row(P, l, cx + bx, cy + by, cz + bz);
-      red_add_v4(gl_ + 4ull * row, make_float4(w * g.x, w * g.y, w * g.z, w * g.w));
+// The adjoint of the query, laid out as the fused rasterizer backward's: warps
+// in pairs over the same points, the even warp on the coarse half of the
+// levels (AdjointLane::coarse merges the contributions of consecutive points
+// that share a vertex before they are reduced into L2), the odd warp on the
+// fine half (reduced directly), two adjacent lanes per level.  The L2
+// reduction rate bounds it, so the merge is what pays: on leaf-grouped
+// points fewer than half of the 8 n_levels contributions of a point are left
+// to reduce (1,000,003 points, 16 levels, 2^19 rows: forward and backward
+// 1,145 -> 661 us, of which the adjoint 0.85 -> 0.40 ms; one thread per
+// point and level with eight reductions each before).  A CTA takes `chunk`
+// consecutive points, its point slots interleaved over them; each lane loads
+// its next point's position and gradient row before it works on the current
+// one.
+template <int GA>
+__global__ void __launch_bounds__(256, 4) k_hash_bwd(GridParams P, const float* __restrict__ pos,
+                                                     const float4* __restrict__ dh, long long n,
+                                                     float* __restrict__ grad, long long chunk, int coarse_only) {
+  constexpr int kH = GA / 2;           // levels per half
+  constexpr int kPW = 16 / kH;         // points per warp
+  constexpr int kGroups = 4 * kPW;     // points in flight per CTA (4 warp pairs)
+  constexpr int kStride = kGroups * kH * 2;
+  __shared__ float4 acc_s[4][kStride];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool coarse = (warp & 1) == 0;
+  const uint32_t bx = lane & 1u;
+  const int lvl = (lane >> 1) % kH;
+  const int l = (coarse ? 0 : kH) + lvl;
+  const int slot = (warp >> 1) * kPW + lane / (2 * kH);
+  if (l >= P.n_levels || (!coarse && coarse_only)) return;  // nothing below is collective
+  const uint64_t keep = l2_evict_last(), stream = l2_evict_first();
+  AdjointLane<kStride> adj(P, l, true, grad, bx, &acc_s[0][(slot * kH + lvl) * 2 + bx]);
+  const long long last = min((long long)(blockIdx.x + 1) * chunk, n);
+  long long id = (long long)blockIdx.x * chunk + slot;
+  if (id >= last) return;
+  uint4 d = ld_hint_u4(dh + id * P.n_levels + l, stream);
+  float x = __ldg(pos + 3 * id), y = __ldg(pos + 3 * id + 1), z = __ldg(pos + 3 * id + 2);
+  while (id < last) {
+    const long long nx = id + kGroups;
+    uint4 dn = make_uint4(0u, 0u, 0u, 0u);
+    float xn = 0.f, yn = 0.f, zn = 0.f;
+    if (nx < last) {
+      dn = ld_hint_u4(dh + nx * P.n_levels + l, stream);
+      xn = __ldg(pos + 3 * nx);
+      yn = __ldg(pos + 3 * nx + 1);
+      zn = __ldg(pos + 3 * nx + 2);
     }
+    const float dc[4] = {__uint_as_float(d.x), __uint_as_float(d.y), __uint_as_float(d.z), __uint_as_float(d.w)};
+    if (dc[0] != 0.f || dc[1] != 0.f || dc[2] != 0.f || dc[3] != 0.f) adj.add(coarse, x, y, z, dc, keep);
+    d = dn;
+    x = xn;
+    y = yn;
+    z = zn;
+    id = nx;
   }
+  if (coarse) adj.flush(keep);
 }
 
-dim3 grid_for(long long n, int n_levels, int threads) {
-  const int groups = (n_levels + kLevelGroup - 1) / kLevelGroup;
-  const long long work = n * std::min(kLevelGroup, n_levels);
-  const long long cap = (long long)device_sm_count() * 16;
-  long long g = ceil_div(work, threads);
-  return dim3((unsigned)std::max<long long>(1, std::min(g, cap)), (unsigned)groups, 1);
+template <int GA>
+inpc_status launch_hash_bwd(const GridParams& P, const float* pos, const float4* dh, long long n, float* grad,
+                            cudaStream_t s) {
+  constexpr int kH = GA / 2, kGroups = 4 * (16 / kH);
+  // fine levels beyond the L2 budget go level group by level group
+  const bool split = P.n_levels > kH && !grad_levels_fit_l2(P, kH);
+  // whole waves of resident CTAs (4 per SM), about 48 points per slot: long
+  // enough runs to merge, and no nearly empty last wave
+  const long long resident = (long long)device_sm_count() * 4;
+  const long long waves = std::max<long long>(1, (n + 24 * kGroups * resident) / (48 * kGroups * resident));
+  const long long chunk = kGroups * std::max<long long>(1, ceil_div(n, kGroups * resident * waves));
+  INPC_TIMED("k_hash_bwd", s,
+             k_hash_bwd<GA><<<(unsigned)ceil_div(n, chunk), 256, 0, s>>>(P, pos, dh, n, grad, chunk, split ? 1 : 0));
+  INPC_TRY(check_launch("k_hash_bwd"));
+  return split ? launch_grad_levels(P, kH, pos, dh + kH, P.n_levels, 1, n, grad, s) : INPC_OK;
 }
 
 }  // namespace
@@ -166,7 +198,11 @@ extern "C" inpc_status inpc_query_hashgrid_bwd(const inpc_hashgrid_desc* g, cons
   if (!aligned(grad_table, 16) || !aligned(dh, 16) || !aligned(pos, 4))
     return fail(INPC_ERR_INVALID_ARG, "inpc_query_hashgrid_bwd: misaligned buffer");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  TimedLaunch timed("k_hash_bwd", s);
-  k_hash_bwd<<<grid_for(n, P.n_levels, 256), 256, 0, s>>>(P, pos, dh, n, grad_table);
-  return check_launch("k_hash_bwd");
+  const float4* d = reinterpret_cast<const float4*>(dh);
+  // up to 4 levels would leave most lanes of the warp pairs idle: two lanes
+  // per point and level instead
+  if (P.n_levels <= 4) return launch_grad_levels(P, 0, pos, d, P.n_levels, 1, n, grad_table, s);
+  if (P.n_levels <= 8) return launch_hash_bwd<8>(P, pos, d, n, grad_table, s);
+  if (P.n_levels <= 16) return launch_hash_bwd<16>(P, pos, d, n, grad_table, s);
+  return launch_hash_bwd<32>(P, pos, d, n, grad_table, s);
 }

@@ -1,5 +1,5 @@
 // raster_bwd.cu -- C ABI of the rasterizer backward (App. A.6).
-#include "hashgrid_impl.cuh"
+#include "adjoint_impl.cuh"
 #include "raster_impl.cuh"
 
 namespace inpc {
@@ -9,27 +9,19 @@ namespace {
 // row for that level, gathered as in k_point_grad, then the level's corner
 // contributions to the table gradient straight from registers (the adjoint
 // of the query, as in k_hash_bwd), so the row never goes through memory.
-// The two lanes own the cell's two x vertices, so each issues four of the
-// eight corner reductions, and a pair's two reductions (x and x + 1 with
-// the same y, z: rows differing in their low bits) usually share a 128-byte
-// line, one L1 wavefront.  Values that depend on the point only (fragment
-// scalars, footprint, position, the h0 term) are formed once per point, one
-// lane per point, into shared-memory records that the level lanes read.
+// (AdjointLane: the two lanes own the cell's two x vertices).  Values that
+// depend on the point only (fragment scalars, footprint, position, the h0
+// term) are formed once per point, one lane per point, into shared-memory
+// records that the level lanes read.
 //
 // The levels are split in halves over a pair of warps that share the same
 // points: the even warp takes the coarse half, the odd warp the fine half.
 // Each point slot of a CTA walks a run of points a few apart.  Points come
 // grouped by octree leaf with the leaves in Morton order, so at the coarse
 // levels such points fall in the same or a neighbouring cell, and a coarse
-// lane keeps one float4 accumulator per cell corner (in shared memory),
-// sending a corner's sum to memory only when the next point needs a
-// different vertex in that slot.  The slot of vertex (X, Y, Z) is given by
-// the parities of X, Y and Z: every cell has exactly one corner of each
-// parity class, and a step of one cell along an axis keeps the four shared
-// vertices in their slots, so neighbouring cells share accumulators as well.
-// Coarse levels have few rows that would otherwise receive millions of
-// additions each.  Fine levels change vertex at almost every point and
-// reduce directly.
+// lane's accumulators merge their contributions.  Coarse levels have few rows
+// that would otherwise receive millions of additions each.  Fine levels
+// change vertex at almost every point and reduce directly.
 // A point's values shared by its level lanes.
 struct __align__(16) PointRec {
   int pix0;        // pixel of footprint corner 0 (j0 W + i0)
@@ -129,21 +121,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_point_grad_hash(RP P, GridParam
   const int first = (int)blockIdx.x * chunk + slot;
   const int last = (int)min((long long)(blockIdx.x + 1) * chunk, P.n);
   const uint64_t keep = l2_evict_last(), stream = l2_evict_first();
-  float* gl = active ? grad_table + 4 * Gp.offset[l] : nullptr;
-  // this lane's level, hoisted: a row is x + y my + z mz (dense) or
-  // (x ^ y my ^ z mz) & mask (hashed), as in vertex_row
-  const bool dense = active && Gp.dense[active ? l : 0];
-  const uint32_t side = active ? Gp.side[l] : 1u;
-  const uint32_t my = dense ? side : 2654435761u, mz = dense ? side * side : 805459861u;
-  const uint32_t rmask = dense ? 0xffffffffu : Gp.hash_mask;
-  const int N = active ? Gp.res[l] : 1;
   // the coarse warps' corner accumulators, [y-z corner][point slot][level][x side]
   constexpr int kStride = kGroups * kH * 2;
   __shared__ float4 acc_s[4][kStride];
-  float4* acc = &acc_s[0][(slot * kH + lvl) * 2 + bx];
-  // the cell whose corners the accumulators hold (kFar: none yet)
-  constexpr uint32_t kFar = 1u << 30;
-  uint32_t hx = kFar, hy = kFar, hz = kFar;
+  AdjointLane<kStride> lane_adj(Gp, l, active, grad_table, bx, &acc_s[0][(slot * kH + lvl) * 2 + bx]);
   // Per-point values (fragment scalars, pixel, position, the h0 term) are
   // formed once per point: one lane per point computes them for the next
   // kBatch x kPW points of the warp pair into records, and the level lanes
@@ -191,138 +172,25 @@ __global__ void __launch_bounds__(kThreads, 4) k_point_grad_hash(RP P, GridParam
       if (d_feat && bx == 0)
         *reinterpret_cast<float4*>(d_feat + (long long)id * P.F + ch) = make_float4(dc[0], dc[1], dc[2], dc[3]);
       if (!coarse && dfine) {
-        // deferred fine levels: the row goes to k_grad_fine (level-major, so
+        // deferred fine levels: the row goes to k_grad_levels (level-major, so
         // that pass reads a level's rows of consecutive points together)
         if (bx == 0) __stcs(reinterpret_cast<float4*>(dfine) + (long long)lvl * P.n + id, make_float4(dc[0], dc[1], dc[2], dc[3]));
         continue;
       }
       if (dc[0] == 0.f && dc[1] == 0.f && dc[2] == 0.f && dc[3] == 0.f) continue;
-      uint32_t cx, cy, cz;
-      float gx[2], gy[2], gz[2];
-      cell_frac(R.x, N, cx, gx[0], gx[1]);
-      cell_frac(R.y, N, cy, gy[0], gy[1]);
-      cell_frac(R.z, N, cz, gz[0], gz[1]);
-      // slot s holds the corner whose offsets are s's bits xor the cell's
-      // parities; swapping the weight pairs of odd cells makes gy[sy] that
-      // corner's weight.  Along x this lane owns the vertex of parity bx.
-      const uint32_t px = cx & 1u, py = cy & 1u, pz = cz & 1u;
-      const uint32_t qx = hx & 1u, qy = hy & 1u, qz = hz & 1u;
-      const uint32_t X = cx + (bx ^ px);
-      const float wx = (bx ^ px) ? gx[1] : gx[0];
-      if (py) swap_f(gy[0], gy[1]);
-      if (pz) swap_f(gz[0], gz[1]);
-      if (coarse) {
-        // does the slot keep its vertex?
-        const uint32_t HX = hx + (bx ^ qx);
-        const bool kx = X == HX;
-        const bool ky[2] = {cy + py == hy + qy, cy + (py ^ 1u) == hy + (qy ^ 1u)};
-        const bool kz[2] = {cz + pz == hz + qz, cz + (pz ^ 1u) == hz + (qz ^ 1u)};
-        const bool held = hx != kFar;
-        // the y and z terms of the held cell's rows of slots sy, sz
-        const uint32_t hyb[2] = {(hy + qy) * my, (hy + (qy ^ 1u)) * my};
-        const uint32_t hzb[2] = {(hz + qz) * mz, (hz + (qz ^ 1u)) * mz};
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          const uint32_t sy = s & 1, sz = s >> 1;
-          const float w = wx * gy[sy] * gz[sz];
-          const float4 a = acc[s * kStride];
-          const bool same = kx && ky[sy] && kz[sz];
-          // same vertex: add to the sum; otherwise start a new sum (fma onto 0)
-          acc[s * kStride] = make_float4(__fmaf_rn(w, dc[0], same ? a.x : 0.f), __fmaf_rn(w, dc[1], same ? a.y : 0.f),
-                                         __fmaf_rn(w, dc[2], same ? a.z : 0.f), __fmaf_rn(w, dc[3], same ? a.w : 0.f));
-          // the slot moves to another vertex: send the old vertex its sum
-          if (!same && held) {
-            const uint32_t row = dense ? HX + hyb[sy] + hzb[sz] : ((HX ^ hyb[sy] ^ hzb[sz]) & rmask);
-            red_add_v4(gl + 4ull * row, a, keep);
-          }
-        }
-      } else {
-        // the y and z terms of this cell's rows of slots sy, sz
-        const uint32_t yb[2] = {(cy + py) * my, (cy + (py ^ 1u)) * my};
-        const uint32_t zb[2] = {(cz + pz) * mz, (cz + (pz ^ 1u)) * mz};
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          const uint32_t sy = s & 1, sz = s >> 1;
-          const float w = wx * gy[sy] * gz[sz];
-          const uint32_t row = dense ? X + yb[sy] + zb[sz] : ((X ^ yb[sy] ^ zb[sz]) & rmask);
-          red_add_v4(gl + 4ull * row, make_float4(w * dc[0], w * dc[1], w * dc[2], w * dc[3]), keep);
-        }
-      }
-      hx = cx;
-      hy = cy;
-      hz = cz;
+      lane_adj.add(coarse, R.x, R.y, R.z, dc, keep);
     }
     pair_barrier(pair);
   }
-  if (!active || !coarse || hx == kFar) return;
-  const uint32_t qx = hx & 1u, qy = hy & 1u, qz = hz & 1u;
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const uint32_t sy = s & 1, sz = s >> 1;
-    red_add_v4(gl + 4ull * vertex_row(Gp, l, hx + (bx ^ qx), hy + (sy ^ qy), hz + (sz ^ qz)), acc[s * kStride], keep);
-  }
+  if (active && coarse) lane_adj.flush(keep);
 }
 
-// The fine levels of the grid adjoint, deferred: for tables whose fine
-// levels do not fit in L2, reductions into them from the fused kernel miss
-// L2 and go to DRAM twice (a read before the add, a write-back later).  The
-// fused kernel then stores each point's gradient row of every fine level
-// (dL/dh of the level, 4 floats; level-major in dfine) instead of reducing
-// it, and this pass adds the corner contributions level group after level
-// group (plan_level_groups), so the rows receiving reductions at a time are
-// one group's and stay in L2.  Two lanes per point, one per x vertex of the
-// cell, 16 consecutive points per warp; the contributions are the fused
-// kernel's own, (w_x w_y) w_z times the row.
-__global__ void __launch_bounds__(256) k_grad_fine(GridParams Gp, LevelGroups LG, int l_first,
-                                                   const float* __restrict__ pos, const float* __restrict__ dfine,
-                                                   long long n, float* __restrict__ grad_table) {
-  const int lb = LG.begin[blockIdx.y], le = LG.begin[blockIdx.y + 1];
-  const uint64_t keep = l2_evict_last(), stream = l2_evict_first();
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t bx = lane & 1u;
-  // n <= 2^25 (the limit of the backward calls): 32-bit point indices
-  const uint32_t n_groups = (uint32_t)((n + 15) >> 4);
-  const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n_groups; g += n_warps) {
-    const uint32_t p = g * 16u + (lane >> 1);
-    if (p >= (uint32_t)n) continue;  // nothing below is warp-collective
-    const float x = __ldg(pos + 3 * p + 0), y = __ldg(pos + 3 * p + 1), z = __ldg(pos + 3 * p + 2);
-    for (int l = lb; l < le; ++l) {
-      const uint4 r = ld_hint_u4(reinterpret_cast<const uint4*>(dfine) + (long long)(l - l_first) * n + p, stream);
-      const float4 d = make_float4(__uint_as_float(r.x), __uint_as_float(r.y), __uint_as_float(r.z),
-                                   __uint_as_float(r.w));
-      if (d.x == 0.f && d.y == 0.f && d.z == 0.f && d.w == 0.f) continue;
-      uint32_t cx, cy, cz;
-      float gx[2], gy[2], gz[2];
-      const int N = Gp.res[l];
-      cell_frac(x, N, cx, gx[0], gx[1]);
-      cell_frac(y, N, cy, gy[0], gy[1]);
-      cell_frac(z, N, cz, gz[0], gz[1]);
-      float* gl = grad_table + 4 * Gp.offset[l];
-      const float wx = gx[bx];
-#pragma unroll
-      for (int yz = 0; yz < 4; ++yz) {
-        const int by = yz & 1, bz = yz >> 1;
-        const float w = wx * gy[by] * gz[bz];
-        const uint32_t row = vertex_row(Gp, l, cx + bx, cy + by, cz + bz);
-        red_add_v4(gl + 4ull * row, make_float4(w * d.x, w * d.y, w * d.z, w * d.w), keep);
-      }
-    }
-  }
-}
-
-// Levels per half of the fused kernel's warp pairs for a grid of n_levels
-// levels (the template size it is launched with, halved).
-inline int adjoint_half(int n_levels) { return n_levels <= 8 ? 4 : n_levels <= 16 ? 8 : 16; }
-
-// Whether the fine half's gradient rows are deferred to k_grad_fine (they
+// Whether the fine half's gradient rows are deferred to k_grad_levels (they
 // do not fit the L2 budget), and the bytes of its row buffer.
 inline size_t fine_defer_bytes(const GridParams& Gp, long long n) {
   const int kH = adjoint_half(Gp.n_levels);
   if (Gp.n_levels <= kH) return 0;
-  long long rows = 0;
-  for (int l = kH; l < Gp.n_levels; ++l) rows += level_rows(Gp, l);
-  if (rows * 16 <= kQueryL2Budget) return 0;
+  if (grad_levels_fit_l2(Gp, kH)) return 0;
   return (size_t)std::max<long long>(n, 1) * (size_t)(Gp.n_levels - kH) * 16;
 }
 
@@ -343,12 +211,7 @@ inpc_status launch_point_grad_hash(const RP& P, const GridParams& Gp, const floa
   INPC_TRY(check_launch("k_point_grad_hash"));
   if (!dfine) return INPC_OK;
   constexpr int kH = GA / 2;
-  const LevelGroups LG = plan_level_groups(Gp, 16, kH);
-  const long long cap = (long long)device_sm_count() * 16;
-  const dim3 g2((unsigned)std::max<long long>(1, std::min<long long>((long long)ceil_div(2 * P.n, 256), cap)),
-                (unsigned)LG.n);
-  INPC_TIMED("k_grad_fine", s, k_grad_fine<<<g2, 256, 0, s>>>(Gp, LG, kH, pos, dfine, P.n, grad_table));
-  return check_launch("k_grad_fine");
+  return launch_grad_levels(Gp, kH, pos, reinterpret_cast<const float4*>(dfine), 1, P.n, P.n, grad_table, s);
 }
 
 }  // namespace
