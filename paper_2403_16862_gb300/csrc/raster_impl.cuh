@@ -1968,60 +1968,91 @@ __global__ void __launch_bounds__(kThreads) k_blend_bwd_heavy(RP P, const FT* __
 }
 
 // ------------------------------------------------------ per-point gradient ---
-// Per point: gather the scalars of its (at most four) splats and the
+// Per point: the scalars of its (at most four) splats and the
 // upstream-gradient rows of their pixels.  d_feat row = sum_k (T_k alpha_k) g_k;
 // d alpha_h = sum_k w_k [unclamped] dL/dalpha_k.
-template <int V, int GA, class FT>
+//
+// A warp takes 32 consecutive points.  First each lane forms one point's
+// scalars (projection, footprint, the four pairs, the opacity path); then the
+// warp goes over the points, GL lanes of V channels per point and 32 / GL
+// points at a time, with the point's scalars from its lane by shuffles: the
+// four row gathers of every point in flight are independent 16-byte loads
+// (where F allows), and the per-point chain (position -> footprint -> rows)
+// is paid once per 32 points.
+template <int V, int GL, class FT>
 __global__ void __launch_bounds__(kThreads) k_point_grad(RP P, const float* __restrict__ pos,
                                                           const float* __restrict__ opacity,
                                                           const FT* __restrict__ feat,
                                                           const float* __restrict__ d_image, RasterWs ws,
                                                           float* __restrict__ d_opacity, float* __restrict__ d_feat) {
-  constexpr int kGroups = kThreads / GA;
-  const Group<GA> G;
-  const int ch = G.lg * V;
-  const bool active = ch < P.F;
-  const long long g0 = (long long)blockIdx.x * kGroups + threadIdx.x / GA;
-  for (long long id = g0; id < P.n; id += (long long)gridDim.x * kGroups) {
-    const uint4 sl = __ldg(reinterpret_cast<const uint4*>(ws.pslot) + id);
-    const uint32_t slots[4] = {sl.x, sl.y, sl.z, sl.w};
-    float dc[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) dc[v] = 0.f;
+  constexpr int kPts = 32 / GL;  // points the warp works on at a time
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int ch = (lane % GL) * V;
+  const int n = (int)P.n;  // <= 2^25 (the limit of the backward calls)
+  const int n_warps = (int)(gridDim.x * blockDim.x) >> 5;
+  for (int b0 = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; 32 * b0 < n; b0 += n_warps) {
+    const int base = 32 * b0;
+    const int id = base + lane;
+    unsigned on = 0;  // bit k: corner k lies on the image
+    int pix0 = 0;     // pixel of corner 0 (may lie outside)
+    float sc[4] = {0.f, 0.f, 0.f, 0.f};
     float dah = 0.f, e_h0 = 0.f;
     Splat s;
-    if ((sl.x & sl.y & sl.z & sl.w) != kNoSlot) {
-      splat_point(P, pos, id, s);
-      const float ah = point_alpha_h(P, opacity, feat, id, &e_h0);
-      float2 sc[4];
+    if (id < n && splat_point(P, pos, id, s)) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) sc[k] = slots[k] == kNoSlot ? make_float2(0.f, 0.f) : __ldg(ws.fscal + 4 * id + k);
+      for (int k = 0; k < 4; ++k)
+        if (corner_pixel(P, s.f, k) >= 0) on |= 1u << k;
+    }
+    if (on) {
+      pix0 = s.f.j0 * P.cam.W + s.f.i0;
+      const float ah = point_alpha_h(P, opacity, feat, id, &e_h0);
+      const float4 f0 = __ldg(reinterpret_cast<const float4*>(ws.fscal) + 2 * (long long)id);
+      const float4 f1 = __ldg(reinterpret_cast<const float4*>(ws.fscal) + 2 * (long long)id + 1);
+      const float da[4] = {f0.y, f0.w, f1.y, f1.w};
+      sc[0] = f0.x; sc[1] = f0.z; sc[2] = f1.x; sc[3] = f1.z;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        if (slots[k] == kNoSlot) continue;
+        if (!((on >> k) & 1u)) continue;
         const float w = corner_weight(s.f, k & 1, k >> 1);
-        if (__fmul_rn(ah, w) <= P.alpha_max) dah = __fmaf_rn(w, sc[k].y, dah);
-        if (active) {
-          const long long pix = (long long)(s.f.j0 + (k >> 1)) * P.cam.W + (s.f.i0 + (k & 1));
-          float g[V];
-          load_vec<V>(d_image + pix * P.F + ch, g);
-#pragma unroll
-          for (int v = 0; v < V; ++v) dc[v] = __fmaf_rn(sc[k].x, g[v], dc[v]);
-        }
+        if (__fmul_rn(ah, w) <= P.alpha_max) dah = __fmaf_rn(w, da[k], dah);
       }
     }
     // head mode: channel 0 of the blended color is the constant 1; the
     // opacity gradient reaches h0 through alpha_h = 1 - exp(-exp(h0))
-    if (P.head && G.lg == 0) dc[0] = dah * (e_h0 * expf(-e_h0));
-    if (active) {
-      float* o = d_feat + id * P.F + ch;
-      if (V == 4) *reinterpret_cast<float4*>(o) = make_float4(dc[0], dc[1], dc[2], dc[3]);
-      else if (V == 2) *reinterpret_cast<float2*>(o) = make_float2(dc[0], dc[1]);
+    const float h0term = P.head ? dah * (e_h0 * expf(-e_h0)) : 0.f;
+    if (!P.head && id < n) d_opacity[id] = dah;
+#pragma unroll 2
+    for (int t = 0; t < GL; ++t) {
+      const int src = t * kPts + lane / GL;
+      const unsigned o = __shfl_sync(full, on, src);
+      const int p0 = __shfl_sync(full, pix0, src);
+      float w[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w[k] = __shfl_sync(full, sc[k], src);
+      const float ht = __shfl_sync(full, h0term, src);
+      if (ch >= P.F || base + src >= n) continue;
+      float g[4][V];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const long long pix = (long long)p0 + (k >> 1) * P.cam.W + (k & 1);
+        if ((o >> k) & 1u) load_vec<V>(d_image + pix * P.F + ch, g[k]);
+      }
+      float dc[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) dc[v] = 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((o >> k) & 1u)
+#pragma unroll
+          for (int v = 0; v < V; ++v) dc[v] = __fmaf_rn(w[k], g[k][v], dc[v]);
+      if (P.head && ch == 0) dc[0] = ht;
+      float* out = d_feat + (long long)(base + src) * P.F + ch;
+      if constexpr (V == 4) *reinterpret_cast<float4*>(out) = make_float4(dc[0], dc[1], dc[2], dc[3]);
       else
 #pragma unroll
-        for (int v = 0; v < V; ++v) o[v] = dc[v];
+        for (int v = 0; v < V; ++v) out[v] = dc[v];
     }
-    if (!P.head && G.lg == 0) d_opacity[id] = dah;
   }
 }
 
@@ -2213,11 +2244,22 @@ inpc_status launch_bwd(const RP& P, const float* pos, const float* opacity, cons
                        const int32_t* n_contrib, const float* d_image, const RasterWs& ws, float* d_opacity,
                        float* d_feat, cudaStream_t s) {
   INPC_TRY((launch_blend_bwd<V, GA, FT>(P, feat, n_contrib, d_image, ws, s)));
-  constexpr int kGroups = kThreads / GA;
-  const long long grid = std::min<long long>(ceil_div(P.n, kGroups), (long long)device_sm_count() * 32);
-  INPC_TIMED("k_point_grad", s,
-             k_point_grad<V, GA, FT><<<(unsigned)std::max<long long>(grid, 1), kThreads, 0, s>>>(
-                 P, pos, opacity, feat, d_image, ws, d_opacity, d_feat));
+  // 16 bytes of the rows per lane where the channel count allows it (rows
+  // are then 16-byte aligned), one channel per lane otherwise (F <= 32)
+  constexpr int kV = V == 1 && GA == 32 ? 1 : 4;
+  const unsigned grid =
+      (unsigned)std::max<long long>(1, std::min<long long>(ceil_div(P.n, kThreads), (long long)device_sm_count() * 16));
+  const auto run = [&](auto kernel) {
+    INPC_TIMED("k_point_grad", s, kernel<<<grid, kThreads, 0, s>>>(P, pos, opacity, feat, d_image, ws, d_opacity, d_feat));
+  };
+  if constexpr (kV == 4) {
+    // F = 64 and 128 run on 16 and 32 lanes of 4 channels
+    run(k_point_grad<4, V == 2 ? 16 : GA, FT>);
+  } else if (P.F == 32) {
+    run(k_point_grad<4, 8, FT>);
+  } else {
+    run(k_point_grad<1, 32, FT>);
+  }
   return check_launch("k_point_grad");
 }
 
