@@ -89,7 +89,7 @@ struct FrontWs {
   uint32_t* done;                  // [3 + 3 V]: W, C, G, then D, S, P of each view
   unsigned long long* cdf_state;   // [Tc] look-back words of the CDF tiles
   unsigned long long* cnt_state;   // [V, Tc] look-back words of the count tiles
-  double* cdf;                     // [L]
+  uint64_t* cdf;                   // [L]
   uint32_t* guide;                 // [2^Gl + 1]
   uint32_t* counts;                // [V, L]
   uint32_t* starts;                // [V, L]
@@ -111,7 +111,7 @@ FrontWs carve_front(void* base, int64_t L, int n_views) {
   w.cnt_state = c.take<unsigned long long>((size_t)Tc * n_views);
   w.counts = c.take<uint32_t>((size_t)L * n_views);
   w.clear_bytes = c.bytes();
-  w.cdf = c.take<double>(L);
+  w.cdf = c.take<uint64_t>(L);
   w.guide = c.take<uint32_t>((int64_t(1) << guide_log2(L)) + 1);
   w.starts = c.take<uint32_t>((size_t)L * n_views);
   w.bytes = c.bytes();
@@ -253,27 +253,22 @@ __global__ void __launch_bounds__(kFrontThreads) k_front(const __grid_constant__
 
     if (st == kStW) {
       // ---- max weight of a tile of leaves (and validation)
-      double m = 0.0;
+      uint64_t m = 0;
       bool bad = false;
       const int64_t i0 = (int64_t)r * kWTile;
-      for (int64_t i = i0 + tid; i < min(L, i0 + kWTile); i += kFrontThreads) {
-        const double x = tree.weights[i];
-        if (!(x >= 0.0) || isinf(x)) bad = true;
-        else m = fmax(m, x);
-      }
-      if (__any_sync(0xffffffffu, bad) && (tid & 31) == 0) raise_status(ws.status, INPC_DEV_BAD_WEIGHT);
-      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if ((tid & 31) == 0 && m > 0.0) atomicMax(ws.wmax, (unsigned long long)__double_as_longlong(m));
+      for (int64_t i = i0 + tid; i < min(L, i0 + kWTile); i += kFrontThreads)
+        weight_max((uint64_t)__double_as_longlong(tree.weights[i]), m, bad);
+      warp_weight_max(m, bad, ws.wmax, ws.status);
       block_signal(ws.done + 0);
     } else if (st == kStC) {
       // ---- quantised weights, exact prefix sum (integers)
       if (!block_wait(ws.done + 0, pl.Tw, pl, ws, &sm.ok)) return;
-      const double wm = __longlong_as_double((long long)__ldcg(ws.wmax));
+      const Quantiser quant(__longlong_as_double((long long)__ldcg(ws.wmax)));
       const int64_t base = (int64_t)r * kScanBlock + (int64_t)tid * kScanItems;
       unsigned long long q[kScanItems], run = 0;
 #pragma unroll
       for (int k = 0; k < kScanItems; ++k) {
-        q[k] = base + k < L ? (unsigned long long)quantised_weight(tree.weights[base + k], wm) : 0ull;
+        q[k] = base + k < L ? (unsigned long long)quant(tree.weights[base + k]) : 0ull;
         run += q[k];
       }
       const unsigned long long pre = scan::block_exclusive_scan<unsigned long long>(run, sm.warp_sums, &sm.total);
@@ -284,17 +279,17 @@ __global__ void __launch_bounds__(kFrontThreads) k_front(const __grid_constant__
 #pragma unroll
       for (int k = 0; k < kScanItems; ++k) {
         acc += q[k];
-        if (base + k < L) ws.cdf[base + k] = (double)acc;
+        if (base + k < L) ws.cdf[base + k] = acc;
       }
       block_signal(ws.done + 1);
     } else if (st == kStG) {
       // ---- guide table
       if (!block_wait(ws.done + 1, pl.Tc, pl, ws, &sm.ok)) return;
-      const double Qd = __ldcg(ws.cdf + L - 1);
-      if (r == 0 && tid == 0 && !(Qd > 0.0)) raise_status(ws.status, INPC_DEV_NO_WEIGHT);
+      const uint64_t Q = __ldcg(ws.cdf + L - 1);
+      if (r == 0 && tid == 0 && Q == 0) raise_status(ws.status, INPC_DEV_NO_WEIGHT);
       const int64_t G1 = (int64_t(1) << pl.Gl) + 1;
       for (int64_t j = (int64_t)r * kScanBlock + tid; j < min(G1, (int64_t)(r + 1) * kScanBlock); j += kFrontThreads)
-        ws.guide[j] = guide_entry(LdL2(), ws.cdf, L, pl.Gl, (uint64_t)Qd, j);
+        ws.guide[j] = guide_entry(LdL2(), ws.cdf, L, pl.Gl, Q, j);
       block_signal(ws.done + 2);
     } else if (st == kStD) {
       // ---- draws of view v -> per-leaf counts
@@ -308,7 +303,7 @@ __global__ void __launch_bounds__(kFrontThreads) k_front(const __grid_constant__
         for (int j = tid; j < L; j += kFrontThreads) sm.vals[j] = 0;
         __syncthreads();
       }
-      const uint64_t Qi = (uint64_t)__ldcg(ws.cdf + L - 1);
+      const uint64_t Qi = __ldcg(ws.cdf + L - 1);
       const int64_t base = (int64_t)tile * kDrawPerCta;
       const int lane = tid & 31;
       for (int k = 0; k < kDrawPerThread; ++k) {
