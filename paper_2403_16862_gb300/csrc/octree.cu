@@ -5,8 +5,9 @@
 // Blending weights: after a forward, every pixel's blended prefix (recorded
 // by the forward in blending order) is walked once more with the forward's
 // own product scan, so T_k alpha_k is bitwise the forward's; each splat's
-// value lands at its bucket slot and a per-point pass combines a point's
-// four splats with their bilinear weights.
+// value lands at its point's entry for the footprint corner it came from
+// and a per-point pass combines a point's four splats with their bilinear
+// weights.
 //
 // Updates: per-leaf max and min of the weights of the points drawn from the
 // leaf (as FP32 bit patterns: non-negative floats order like their bits)
@@ -30,18 +31,19 @@ __global__ void __launch_bounds__(256) k_pixel_splat_weights(RP P, const int32_t
     const uint32_t s0 = ws.pix_start[q];
     const int m = (int)(ws.pix_start[q + 1] - s0);
     const int nb = m > 0 ? blended_count(n_contrib, q, m) : 0;
+    const int qy = (int)(q / P.cam.W), qx = (int)(q - (long long)qy * P.cam.W);
     float T = 1.0f;
     for (int b = 0; b < nb; b += 32) {
       const bool valid = b + G.lg < nb;
-      uint32_t slot = 0;
+      uint32_t id = 0;
       float a = 0.f;
       if (valid) {
         const uint2 o = order_at(P, ws, s0, m, b + G.lg);
-        slot = o.x;
+        id = o.y;
         a = ws.alpha[s0 + o.x];
       }
       const ChunkT<32> ct = chunk_transmittance<32>(G, P, a, valid, min(32, nb - b), T);
-      if (G.lg < ct.take) reinterpret_cast<float*>(ws.fscal + s0 + slot)[0] = __fmul_rn(ct.Tk, a);
+      if (G.lg < ct.take) reinterpret_cast<float*>(ws.fscal + frag_index(ws, id, qx, qy))[0] = __fmul_rn(ct.Tk, a);
       T = G.bcast(ct.Tn, ct.take - 1);
       if (ct.stop) break;
     }
@@ -52,15 +54,15 @@ __global__ void __launch_bounds__(256) k_point_blend_weights(RP P, const float* 
                                                             float* __restrict__ b_out) {
   for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < P.n;
        id += (long long)gridDim.x * blockDim.x) {
-    const uint4 sl = __ldg(reinterpret_cast<const uint4*>(ws.pslot) + id);
-    const uint32_t slots[4] = {sl.x, sl.y, sl.z, sl.w};
     float b = 0.f;
-    if ((sl.x & sl.y & sl.z & sl.w) != kNoSlot) {
-      Splat s;
-      splat_point(P, pos, id, s);
+    Splat s;
+    if (splat_point(P, pos, id, s)) {
+      // zero where nothing blended
+      const float4 f0 = __ldg(reinterpret_cast<const float4*>(ws.fscal) + 2 * id);
+      const float4 f1 = __ldg(reinterpret_cast<const float4*>(ws.fscal) + 2 * id + 1);
+      const float sc[4] = {f0.x, f0.z, f1.x, f1.z};
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (slots[k] != kNoSlot) b = __fmaf_rn(corner_weight(s.f, k & 1, k >> 1), ws.fscal[slots[k]].x, b);
+      for (int k = 0; k < 4; ++k) b = __fmaf_rn(corner_weight(s.f, k & 1, k >> 1), sc[k], b);
     }
     b_out[id] = b;
   }

@@ -3,8 +3,8 @@
 //
 // Ordering.  Algorithm 1 sorts all splats globally by (pixel, depth).  Here
 // the pixel is the most significant radix digit and is handled by a
-// counting sort into per-pixel buckets (k_pix_count, prefix sum,
-// k_pix_scatter); each bucket is then ordered by the remaining key
+// counting sort into per-pixel buckets (raster_bin.cuh: k_pix_count, prefix
+// sum, k_pix_scatter); each bucket is then ordered by the remaining key
 // (depth field << idb | point index) by the threads that blend it: in
 // registers by a group of GA lanes per pixel for buckets of at most
 // GA * kRegMax fragments (on 32-bit keys relative to the bucket's nearest
@@ -59,7 +59,6 @@ constexpr int kIdBits = 25;
 constexpr int kKeyBits = 56;
 constexpr int64_t kMaxFwdPoints = int64_t(1) << 28;  // 4n fragment slots stay below 2^32
 constexpr int kHeavyKeys = 2048;  // shared-memory bucket entries on the CTA path (larger buckets sort in global memory)
-constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
 
 struct RP {
   Cam cam;
@@ -90,12 +89,10 @@ struct RasterWs {
   uint32_t* large;           // [n_pix] pixels with 4 or 8 registers per lane
   unsigned long long* keys;  // [4n] bucketed fragment keys
   float* alpha;              // [4n] fragment alphas
-  uint32_t* pslot;           // [4n] bucket slot of each point corner (kNoSlot off-image)
   uint32_t* porg;            // [n] footprint origin of each point: (i0 + 1) | (j0 + 1) << 16
   float* pexp;               // [n] exp(h0) of each point (head mode)
   float2* fscal;             // [4n] backward per-fragment scalars, point-major: entry 4 p + c is point p's
-                             // footprint corner c (the per-point blending weights keep their own slot-major
-                             // values here)
+                             // footprint corner c (also the per-point blending weights' values)
   unsigned long long* ka;    // [4n] global-sort result (largest buckets only)
   uint32_t* va;
   unsigned long long* kb;    // [4n] global-sort scratch, then per-fragment (T_k, c_k . g)
@@ -122,7 +119,6 @@ RasterWs carve(void* base, long long n_pix, long long n) {
   w.large = c.take<uint32_t>(n_pix);
   w.keys = c.take<unsigned long long>(nf);
   w.alpha = c.take<float>(nf);
-  w.pslot = c.take<uint32_t>(nf);
   w.porg = c.take<uint32_t>(std::max<long long>(n, 1));
   w.pexp = c.take<float>(std::max<long long>(n, 1));
   w.fscal = c.take<float2>(nf);
@@ -187,133 +183,13 @@ __device__ __forceinline__ float alpha_input(const RP& P, const float* __restric
   return P.head ? ld1(feat + (long long)P.F * id) : __ldg(opacity + id);
 }
 
-// Warp aggregation of the per-pixel counters: points come grouped by leaf,
-// so consecutive lanes often hit the same pixel.  A run of equal pixels over
-// consecutive lanes is found with one shuffle and one ballot (its start is a
-// lane whose pixel differs from the previous lane's), and its first lane
-// updates the counter for the whole run.
-struct LaneRun {
-  int start;  // first lane of this lane's run
-  int len;    // lanes in the run (valid in the first lane)
-};
+}  // namespace
+}  // namespace inpc
 
-__device__ __forceinline__ LaneRun lane_run(int q, int lane) {
-  const int prev = __shfl_up_sync(0xffffffffu, q, 1);
-  const unsigned starts = __ballot_sync(0xffffffffu, lane == 0 || prev != q);
-  const unsigned upto = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);
-  const unsigned later = starts & ~upto;
-  LaneRun r;
-  r.start = 31 - __clz(starts & upto);
-  r.len = (later ? __ffs(later) - 1 : 32) - lane;
-  return r;
-}
+#include "raster_bin.cuh"
 
-__global__ void __launch_bounds__(256) k_pix_count(RP P, const float* __restrict__ pos,
-                                                   uint32_t* __restrict__ pix_count) {
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int n = (int)P.n;  // <= 2^28
-  const int stride = gridDim.x * blockDim.x;
-  // each iteration loads the next point's position while it bins this one
-  float x = 0.f, y = 0.f, z = 0.f;
-  if (blockIdx.x * blockDim.x + threadIdx.x < n) {
-    const long long id = blockIdx.x * blockDim.x + threadIdx.x;
-    x = __ldg(pos + 3 * id); y = __ldg(pos + 3 * id + 1); z = __ldg(pos + 3 * id + 2);
-  }
-  for (int base = blockIdx.x * blockDim.x; base < n; base += stride) {
-    const int id = base + threadIdx.x;
-    const long long nid = (long long)id + stride;
-    float nx = 0.f, ny = 0.f, nz = 0.f;
-    if (nid < n) {
-      nx = __ldg(pos + 3 * nid); ny = __ldg(pos + 3 * nid + 1); nz = __ldg(pos + 3 * nid + 2);
-    }
-    int q[4] = {-1, -1, -1, -1};
-    Splat s;
-    if (id < n && splat_xyz(P, x, y, z, s))
-      for (int k = 0; k < 4; ++k) q[k] = corner_pixel(P, s.f, k);
-    x = nx; y = ny; z = nz;
-    for (int k = 0; k < 4; ++k) {
-      const LaneRun run = lane_run(q[k], lane);
-      if (q[k] >= 0 && run.start == lane) atomicAdd(pix_count + q[k], (uint32_t)run.len);
-    }
-  }
-}
-
-template <class FT>
-__global__ void __launch_bounds__(256) k_pix_scatter(RP P, const float* __restrict__ pos,
-                                                     const float* __restrict__ opacity,
-                                                     const FT* __restrict__ feat,
-                                                     const uint32_t* __restrict__ pix_start,
-                                                     uint32_t* __restrict__ pix_count,
-                                                     unsigned long long* __restrict__ keys,
-                                                     float* __restrict__ alpha, uint32_t* __restrict__ pslot,
-                                                     uint32_t* __restrict__ porg, float* __restrict__ pexp) {
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int n = (int)P.n;  // <= 2^28
-  const int stride = gridDim.x * blockDim.x;
-  // each iteration loads the next point's position and alpha input while it
-  // bins this one, so those round trips overlap this point's atomics
-  float x = 0.f, y = 0.f, z = 0.f, av = 0.f;
-  if (blockIdx.x * blockDim.x + threadIdx.x < n) {
-    const long long id = blockIdx.x * blockDim.x + threadIdx.x;
-    x = __ldg(pos + 3 * id); y = __ldg(pos + 3 * id + 1); z = __ldg(pos + 3 * id + 2);
-    av = alpha_input(P, opacity, feat, id);
-  }
-  for (int base = blockIdx.x * blockDim.x; base < n; base += stride) {
-    const int id = base + threadIdx.x;
-    const long long nid = (long long)id + stride;
-    float nx = 0.f, ny = 0.f, nz = 0.f, na = 0.f;
-    if (nid < n) {
-      nx = __ldg(pos + 3 * nid); ny = __ldg(pos + 3 * nid + 1); nz = __ldg(pos + 3 * nid + 2);
-      na = alpha_input(P, opacity, feat, nid);
-    }
-    int q[4] = {-1, -1, -1, -1};
-    Splat s;
-    float ah = 0.f;
-    bool splat_ok = false;
-    float e_h0 = 0.f;
-    if (id < n && splat_xyz(P, x, y, z, s)) {
-      for (int k = 0; k < 4; ++k) q[k] = corner_pixel(P, s.f, k);
-      // head mode: alpha_h = 1 - exp(-exp(h0)) as in point_alpha_h, with
-      // exp(h0) kept for the backward's opacity path
-      e_h0 = P.head ? expf(av) : 0.f;
-      ah = P.head ? -expm1f(-e_h0) : av;
-      splat_ok = true;
-    }
-    x = nx; y = ny; z = nz; av = na;
-    const unsigned long long key = ((unsigned long long)(__float_as_uint(s.d) - P.dbase) << P.idb) | (unsigned long long)id;
-    // the four corners' bucket offsets and atomics are all issued before
-    // any result is used, so their round trips overlap
-    LaneRun run[4];
-    uint32_t start[4], top[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      run[k] = lane_run(q[k], lane);
-      start[k] = q[k] >= 0 ? __ldg(pix_start + q[k]) : 0u;
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      // counts run down from the bucket size, so the buckets fill back to front
-      top[k] = 0;
-      if (q[k] >= 0 && run[k].start == lane) top[k] = atomicSub(pix_count + q[k], (uint32_t)run[k].len);
-    }
-    uint32_t slots[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint32_t t = __shfl_sync(full, top[k], run[k].start);
-      slots[k] = kNoSlot;
-      if (q[k] >= 0) {
-        slots[k] = start[k] + t - 1 - (uint32_t)(lane - run[k].start);
-        keys[slots[k]] = key;
-        alpha[slots[k]] = fminf(__fmul_rn(ah, corner_weight(s.f, k & 1, k >> 1)), P.alpha_max);
-      }
-    }
-    if (id < n) reinterpret_cast<uint4*>(pslot)[id] = make_uint4(slots[0], slots[1], slots[2], slots[3]);
-    if (id < n) porg[id] = splat_ok ? ((uint32_t)(s.f.i0 + 1) & 0xffffu) | ((uint32_t)(s.f.j0 + 1) << 16) : 0u;
-    if (id < n && P.head) pexp[id] = e_h0;
-  }
-}
+namespace inpc {
+namespace {
 
 struct CountLoad {
   const uint32_t* c;
@@ -2166,16 +2042,50 @@ inpc_status set_smem(K kernel, size_t bytes, SmemOnce& once) {
   return INPC_OK;
 }
 
+// Counting pass: chunks of kT kPP points.
+template <int kT, int kPP>
+inpc_status launch_count(const RP& P, const float* pos, const RasterWs& ws, cudaStream_t s) {
+  const long long chunks = ceil_div(P.n, kT * kPP), resident = (long long)device_sm_count() * (2048 / kT);
+  INPC_TIMED("k_pix_count", s,
+             k_pix_count<kT, kPP><<<(unsigned)std::min(chunks, resident), kT, 0, s>>>(P, pos, ws.pix_count));
+  return check_launch("k_pix_count");
+}
+
+// The window pays in the scattering pass where a chunk's pixels get several
+// fragments each and the chunks (1,024 points; two CTAs of 512 threads per
+// SM) fill the GPU several times over.  Measured, window against direct: 252
+// fragments a pixel (67M points) 3.74 and 5.68 ms, 16 (4M) 346 and 382 us, 15
+// (1M) 78 and 66 us, 4 (1M) 138 and 81 us.
+template <class FT>
+inpc_status launch_scatter(const RP& P, const float* pos, const float* opacity, const FT* feat, const RasterWs& ws,
+                           cudaStream_t s) {
+  constexpr int kT = 512, kPP = 2;
+  const long long chunks = ceil_div(P.n, kT * kPP), resident = (long long)device_sm_count() * 2;
+  if (chunks >= 6 * resident && 4 * P.n >= 12 * P.n_pix) {
+    constexpr size_t smem = sizeof(ScatterSmem<kT, kPP>);
+    static SmemOnce once;
+    INPC_TRY(set_smem(k_pix_scatter<kT, kPP, FT>, smem, once));
+    INPC_TIMED("k_pix_scatter", s,
+               k_pix_scatter<kT, kPP, FT><<<(unsigned)resident, kT, smem, s>>>(P, pos, opacity, feat, ws));
+  } else {
+    INPC_TIMED("k_pix_scatter", s,
+               k_pix_scatter_direct<FT><<<point_grid(P.n), 256, 0, s>>>(P, pos, opacity, feat, ws.pix_start,
+                                                                        ws.pix_count, ws.keys, ws.alpha, ws.porg,
+                                                                        ws.pexp));
+  }
+  return check_launch("k_pix_scatter");
+}
+
 // Forward binning: per-pixel counts, offsets, buckets (keys and alphas),
-// per-point slots and the list of pixels for the CTA path (all kept in the
-// workspace for the backward).
+// per-point footprint origins and the list of pixels for the CTA path (all
+// kept in the workspace for the backward).
 template <class FT>
 inpc_status bin_fragments(const RP& P, const float* pos, const float* opacity, const FT* feat, const RasterWs& ws,
                           uint32_t cap_small, uint32_t cap_group, cudaStream_t s) {
   INPC_CUDA(cudaMemsetAsync(ws.pix_count, 0, sizeof(uint32_t) * P.n_pix, s), "clear pixel counts");
   if (P.n > 0) {
-    INPC_TIMED("k_pix_count", s, k_pix_count<<<point_grid(P.n), 256, 0, s>>>(P, pos, ws.pix_count));
-    INPC_TRY(check_launch("k_pix_count"));
+    INPC_TRY(P.n >= (long long)device_sm_count() * 2048 ? (launch_count<512, 2>(P, pos, ws, s))
+                                                        : (launch_count<256, 1>(P, pos, ws, s)));
   }
   INPC_TRY((scan::run<uint32_t, CountLoad, false>(CountLoad{ws.pix_count}, P.n_pix, ws.pix_start, ws.tops, s)));
   const long long nb = ceil_div(P.n_pix, scan::kBlock);
@@ -2184,10 +2094,7 @@ inpc_status bin_fragments(const RP& P, const float* pos, const float* opacity, c
                                                                ws.pix_start, 4 * (cap_small / 2), ws.wide_count);
   INPC_TRY(check_launch("k_classify"));
   if (P.n > 0) {
-    INPC_TIMED("k_pix_scatter", s,
-               k_pix_scatter<FT><<<point_grid(P.n), 256, 0, s>>>(P, pos, opacity, feat, ws.pix_start, ws.pix_count,
-                                                                 ws.keys, ws.alpha, ws.pslot, ws.porg, ws.pexp));
-    INPC_TRY(check_launch("k_pix_scatter"));
+    INPC_TRY(launch_scatter<FT>(P, pos, opacity, feat, ws, s));
   }
   return INPC_OK;
 }
