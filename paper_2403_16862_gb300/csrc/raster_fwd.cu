@@ -1,4 +1,5 @@
 // raster_fwd.cu -- C ABI of the rasterizer forward (Sec. 3.4, Algorithm 1).
+#include "raster_fwd.h"
 #include "raster_impl.cuh"
 
 using namespace inpc;
@@ -31,17 +32,12 @@ extern "C" inpc_status inpc_rasterize_fwd(const inpc_camera* cam, const inpc_ras
   if (!aligned(feat, va) || !aligned(image, va) || !aligned(pos, 4))
     return fail(INPC_ERR_INVALID_ARG, "feat/image must be %zu-byte aligned", va);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  RasterWs ws = carve(workspace, P.n_pix, n);
-  INPC_CUDA(cudaMemsetAsync(workspace, 0, kHeaderBytes, s), "clear header");
-  return dispatch(P.F, [&](auto Vc, auto Gc) {
-    constexpr int V = decltype(Vc)::value, GA = decltype(Gc)::value;
-    if constexpr (GA != 32) {
-      if (P.bf16) return fail(INPC_ERR_UNSUPPORTED, "BF16 features need n_channels = 32, 64 or 128");
-    } else if (P.bf16)
-      return launch_fwd<V, GA, __nv_bfloat16>(P, pos, opacity, static_cast<const __nv_bfloat16*>(feat), ws,
-                                              static_cast<__nv_bfloat16*>(image), T_final, n_contrib, s);
-    return launch_fwd<V, GA, float>(P, pos, opacity, static_cast<const float*>(feat), ws, static_cast<float*>(image),
-                                    T_final, n_contrib, s);
+  const RasterFwdCall call{cam, opts, pos, opacity, feat, n, image, T_final, n_contrib, workspace, s};
+  return dispatch(P.F, [&](auto, auto Gc) -> inpc_status {
+    constexpr int GA = decltype(Gc)::value;
+    if (P.bf16 && GA != 32) return fail(INPC_ERR_UNSUPPORTED, "BF16 features need n_channels = 32, 64 or 128");
+    INPC_CUDA(cudaMemsetAsync(workspace, 0, kHeaderBytes, s), "clear header");
+    if (P.bf16) return raster_fwd_bf16(call);
+    return GA <= 4 ? raster_fwd_narrow4(call) : GA < 32 ? raster_fwd_narrow16(call) : raster_fwd_wide(call);
   });
 }
-

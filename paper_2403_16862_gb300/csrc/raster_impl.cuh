@@ -8,7 +8,8 @@
 // (depth field << idb | point index) by the threads that blend it: in
 // registers by a group of GA lanes per pixel for buckets of at most
 // GA * kRegMax fragments (on 32-bit keys relative to the bucket's nearest
-// depth whenever those order it exactly); by a CTA for larger ones, which
+// depth whenever those order it exactly); by one warp up to kWarpKeys
+// (raster_warp.cuh); by a CTA for larger ones, which
 // first selects the nearest fragments by a depth histogram and has one warp
 // sort them in registers, and falls back to a shared-memory bitonic network
 // or, beyond the shared-memory capacity, a stable LSD radix sort in global
@@ -58,6 +59,8 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kIdBits = 25;
 constexpr int kKeyBits = 56;
 constexpr int64_t kMaxFwdPoints = int64_t(1) << 28;  // 4n fragment slots stay below 2^32
+constexpr int kCandMax = 256;    // fragments that one warp sorts at most
+constexpr int kWarpKeys = 1024;  // bucket size up to which one warp selects the nearest fragments
 constexpr int kHeavyKeys = 2048;  // shared-memory bucket entries on the CTA path (larger buckets sort in global memory)
 
 struct RP {
@@ -82,11 +85,15 @@ struct RasterWs {
   uint32_t* heavy_next;      // header word 4: the forward CTA kernel's next list entry
   uint32_t* wide_count;      // header word 5: forward list entries with 8 registers per lane (at the list's end)
   uint32_t* wide_next;       // header word 6: their cursor
+  uint32_t* select_count;    // header word 7: pixels with a selection by one warp (the front of mid)
+  uint32_t* warp_count;      // header word 8: pixels with a whole bucket for one warp (the back of mid)
+  uint32_t* warp_next;       // header word 9: the cursor over both
   uint32_t* pix_count;       // [n_pix]
   uint32_t* pix_start;       // [n_pix + 1]
   uint32_t* tops;            // prefix-sum block totals
   uint32_t* heavy;           // [n_pix] pixels on the CTA path
   uint32_t* large;           // [n_pix] pixels with 4 or 8 registers per lane
+  uint32_t* mid;             // [n_pix] pixels blended by one warp each (raster_warp.cuh)
   unsigned long long* keys;  // [4n] bucketed fragment keys
   float* alpha;              // [4n] fragment alphas
   uint32_t* porg;            // [n] footprint origin of each point: (i0 + 1) | (j0 + 1) << 16
@@ -111,12 +118,16 @@ RasterWs carve(void* base, long long n_pix, long long n) {
   w.heavy_next = base ? reinterpret_cast<uint32_t*>(base) + 4 : nullptr;
   w.wide_count = base ? reinterpret_cast<uint32_t*>(base) + 5 : nullptr;
   w.wide_next = base ? reinterpret_cast<uint32_t*>(base) + 6 : nullptr;
+  w.select_count = base ? reinterpret_cast<uint32_t*>(base) + 7 : nullptr;
+  w.warp_count = base ? reinterpret_cast<uint32_t*>(base) + 8 : nullptr;
+  w.warp_next = base ? reinterpret_cast<uint32_t*>(base) + 9 : nullptr;
   const long long nf = std::max<long long>(4 * n, 1);
   w.pix_count = c.take<uint32_t>(n_pix);
   w.pix_start = c.take<uint32_t>(n_pix + 1);
   w.tops = c.take<uint32_t>(scan::n_tops(n_pix));
   w.heavy = c.take<uint32_t>(n_pix);
   w.large = c.take<uint32_t>(n_pix);
+  w.mid = c.take<uint32_t>(n_pix);
   w.keys = c.take<unsigned long long>(nf);
   w.alpha = c.take<float>(nf);
   w.porg = c.take<uint32_t>(std::max<long long>(n, 1));
@@ -201,19 +212,26 @@ struct CountLoad {
 // the list of the register kernel with 4 registers per lane, up to
 // cap_large to its back, for the kernel with 8 (two kernels, each with half
 // the code: the unrolled sorting networks of both sizes in one kernel
-// stalled it on instruction fetch); larger ones go to the CTA path.
-__global__ void k_classify(const uint32_t* __restrict__ pix_start, long long n_pix, const uint32_t* __restrict__ tops,
-                           long long nb, uint32_t cap_small, uint32_t cap_large, uint32_t* __restrict__ heavy,
-                           uint32_t* heavy_count, uint32_t* __restrict__ large, uint32_t* large_count,
-                           uint32_t* __restrict__ pix_start_w, uint32_t cap_mid, uint32_t* wide_count) {
+// stalled it on instruction fetch); up to kCandMax (where cap_large is
+// below that) and up to kWarpKeys one warp takes a pixel (raster_warp.cuh);
+// larger ones go to the CTA path.
+struct ClassCaps {
+  uint32_t small, mid, large;
+};
+
+__global__ void k_classify(long long n_pix, long long nb, ClassCaps cap, RasterWs ws) {
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (q == 0) pix_start_w[n_pix] = tops[nb];
+  const uint32_t* pix_start = ws.pix_start;
+  if (q == 0) ws.pix_start[n_pix] = ws.tops[nb];
   if (q >= n_pix) return;
-  const uint32_t end = q + 1 < n_pix ? pix_start[q + 1] : tops[nb];
+  const uint32_t end = q + 1 < n_pix ? pix_start[q + 1] : ws.tops[nb];
   const uint32_t m = end - pix_start[q];
-  if (m > cap_large) heavy[atomicAdd(heavy_count, 1u)] = (uint32_t)q;
-  else if (m > cap_mid) large[n_pix - 1 - atomicAdd(wide_count, 1u)] = (uint32_t)q;
-  else if (m > cap_small) large[atomicAdd(large_count, 1u)] = (uint32_t)q;
+  if (m <= cap.small) return;
+  if (m <= cap.mid) ws.large[atomicAdd(ws.large_count, 1u)] = (uint32_t)q;
+  else if (m <= cap.large) ws.large[n_pix - 1 - atomicAdd(ws.wide_count, 1u)] = (uint32_t)q;
+  else if (m <= (uint32_t)kCandMax) ws.mid[n_pix - 1 - atomicAdd(ws.warp_count, 1u)] = (uint32_t)q;
+  else if (m <= (uint32_t)kWarpKeys) ws.mid[atomicAdd(ws.select_count, 1u)] = (uint32_t)q;
+  else ws.heavy[atomicAdd(ws.heavy_count, 1u)] = (uint32_t)q;
 }
 
 // Backward classes by blended count (the forward's n_contrib, clamped to the
@@ -813,6 +831,55 @@ __device__ __forceinline__ void prefetch_row64(const FT* __restrict__ feat, uint
   for (int k = 0; k < (int)(64 * sizeof(FT)) / 128; ++k) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 128 * k));
 }
 
+// Adds wk c of a chunk's fragments (lane j: fragment j's point and weight;
+// the first `take`) to the lane's 16 channels of its slot.
+template <class FT>
+__device__ __forceinline__ void slots_gather(const Group<32>& G, const RP& P, const FT* __restrict__ feat, uint32_t id,
+                                             float wk, int take, float (&acc)[16]) {
+  const int q = G.lg & 3, f = G.lg >> 2;
+#pragma unroll 2
+  for (int p = 0; p * 8 < take; ++p) {
+    const int j = 8 * p + f;
+    const uint32_t idj = __shfl_sync(0xffffffffu, id, j);
+    const float wj = __shfl_sync(0xffffffffu, wk, j);
+    if (j < take) {
+      float c[16];
+      Slot64<FT>::load(feat + 64ll * idj, q, c);
+      if (P.head && q == 0) c[0] = 1.0f;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) acc[e] = __fmaf_rn(wj, c[e], acc[e]);
+    }
+  }
+}
+
+// Reduce-scatters the slots' sums (lane bits 4, 3, 2) and writes the pixel.
+template <class FT>
+__device__ __forceinline__ void slots_write(const Group<32>& G, const float (&acc)[16], long long pix,
+                                            FT* __restrict__ image) {
+  const int q = G.lg & 3;
+  const int h4 = (G.lg >> 4) & 1, h3 = (G.lg >> 3) & 1, h2 = (G.lg >> 2) & 1;
+  float r8[8], r4[4], r2[2];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float send = h4 ? acc[k] : acc[8 + k];
+    const float keep = h4 ? acc[8 + k] : acc[k];
+    r8[k] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, 16));
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float send = h3 ? r8[k] : r8[4 + k];
+    const float keep = h3 ? r8[4 + k] : r8[k];
+    r4[k] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, 8));
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float send = h2 ? r4[k] : r4[2 + k];
+    const float keep = h2 ? r4[2 + k] : r4[k];
+    r2[k] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, 4));
+  }
+  Slot64<FT>::store2(image + pix * 64, Slot64<FT>::channel(q, 8 * h4 + 4 * h3 + 2 * h2), r2[0], r2[1]);
+}
+
 template <class FT, int R>
 __device__ void blend_fwd_slots(const Group<32>& G, const RP& P, const RasterWs& ws, uint32_t s0, int m,
                                 long long pix, const FT* __restrict__ feat, FT* __restrict__ image,
@@ -853,7 +920,6 @@ __device__ void blend_fwd_slots(const Group<32>& G, const RP& P, const RasterWs&
       a_sorted[r] = (R == 2 && (pos >> 5) == 1) ? v1 : v0;
     }
   }
-  const int q = G.lg & 3, f = G.lg >> 2;
   float acc[16];
 #pragma unroll
   for (int e = 0; e < 16; ++e) acc[e] = 0.f;
@@ -871,46 +937,12 @@ __device__ void blend_fwd_slots(const Group<32>& G, const RP& P, const RasterWs&
     const ChunkT<32> ct = chunk_transmittance<32>(G, P, a, valid, min(32, m - b), T);
     const float wk = __fmul_rn(ct.Tk, a);
     if (G.lg < ct.take) ws.order[s0 + b + G.lg] = make_uint2(reg_pos(key[r]), id);
-#pragma unroll 2
-    for (int p = 0; p * 8 < ct.take; ++p) {
-      const int j = 8 * p + f;
-      const uint32_t idj = __shfl_sync(0xffffffffu, id, j);
-      const float wj = __shfl_sync(0xffffffffu, wk, j);
-      if (j < ct.take) {
-        float c[16];
-        Slot64<FT>::load(feat + 64ll * idj, q, c);
-        if (P.head && q == 0) c[0] = 1.0f;
-#pragma unroll
-        for (int e = 0; e < 16; ++e) acc[e] = __fmaf_rn(wj, c[e], acc[e]);
-      }
-    }
+    slots_gather(G, P, feat, id, wk, ct.take, acc);
     cnt += ct.take;
     T = G.bcast(ct.Tn, ct.take - 1);
     if (ct.stop) break;
   }
-  // reduce-scatter over the 8 slots (lane bits 4, 3, 2)
-  const int h4 = (G.lg >> 4) & 1, h3 = (G.lg >> 3) & 1, h2 = (G.lg >> 2) & 1;
-  float r8[8], r4[4], r2[2];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float send = h4 ? acc[k] : acc[8 + k];
-    const float keep = h4 ? acc[8 + k] : acc[k];
-    r8[k] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, 16));
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float send = h3 ? r8[k] : r8[4 + k];
-    const float keep = h3 ? r8[4 + k] : r8[k];
-    r4[k] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, 8));
-  }
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const float send = h2 ? r4[k] : r4[2 + k];
-    const float keep = h2 ? r4[2 + k] : r4[k];
-    r2[k] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, 4));
-  }
-  const int e0 = 8 * h4 + 4 * h3 + 2 * h2;
-  Slot64<FT>::store2(image + pix * 64, Slot64<FT>::channel(q, e0), r2[0], r2[1]);
+  slots_write(G, acc, pix, image);
   if (G.lg == 0) {
     T_final[pix] = T;
     n_contrib[pix] = cnt;
@@ -1265,11 +1297,19 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_bwd(RP P, const FT* __res
   }
 }
 
+}  // namespace
+}  // namespace inpc
+
+#include "raster_warp.cuh"
+
+namespace inpc {
+namespace {
+
 template <int V, int GA, class FT>
 __global__ void __launch_bounds__(kThreads, 3) k_blend_bwd_large(RP P, const FT* __restrict__ feat,
                                                                const int32_t* __restrict__ n_contrib,
                                                                const float* __restrict__ d_image, RasterWs ws) {
-  const Group<GA> G;
+  const Group<32> G;  // one warp per pixel
   const uint32_t n_large = *ws.large_count;
   // as in the forward list kernel, each group takes the next pixel when done
   for (;;) {
@@ -1281,8 +1321,14 @@ __global__ void __launch_bounds__(kThreads, 3) k_blend_bwd_large(RP P, const FT*
     const uint32_t s0 = ws.pix_start[q];
     const int m = (int)(ws.pix_start[q + 1] - s0);
     const int nb = blended_count(n_contrib, q, m);
-    if (nb <= 4 * GA) blend_bwd_reg<V, GA, FT, 4>(G, P, ws, s0, m, nb, q, feat, d_image);
-    else blend_bwd_reg<V, GA, FT, kRegMax>(G, P, ws, s0, m, nb, q, feat, d_image);
+    if constexpr (GA < 32) {
+      if (nb <= 64) blend_bwd_warp<V, GA, FT, 2>(G, P, ws, s0, m, nb, q, feat, d_image);
+      else if (nb <= 128) blend_bwd_warp<V, GA, FT, 4>(G, P, ws, s0, m, nb, q, feat, d_image);
+      else blend_bwd_warp<V, GA, FT, 8>(G, P, ws, s0, m, nb, q, feat, d_image);
+    } else {
+      if (nb <= 4 * GA) blend_bwd_reg<V, GA, FT, 4>(G, P, ws, s0, m, nb, q, feat, d_image);
+      else blend_bwd_reg<V, GA, FT, kRegMax>(G, P, ws, s0, m, nb, q, feat, d_image);
+    }
   }
 }
 
@@ -1735,7 +1781,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_fwd_heavy(RP P, const FT*
   __shared__ SelSmem X;
   const HeavyBuf B(dyn);
   __shared__ uint32_t next;
-  const uint32_t n_heavy = *ws.heavy_count;
+  // the largest buckets and what the warps left open, then the buckets of up
+  // to kWarpKeys where these are few
+  const uint32_t n_big = *ws.heavy_count, n_mid = *ws.select_count;
+  const uint32_t n_heavy = n_big + (n_mid < kSelectMin ? n_mid : 0u);
   // the CTA takes the next pixel of the list when it is done with one; every
   // iteration ends with a barrier, so `next` is read before it is rewritten
   for (;;) {
@@ -1743,7 +1792,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_fwd_heavy(RP P, const FT*
     __syncthreads();
     const uint32_t h = next;
     if (h >= n_heavy) break;
-    const long long q = ws.heavy[h];
+    const long long q = h < n_big ? ws.heavy[h] : ws.mid[h - n_big];
     const uint32_t s0 = ws.pix_start[q];
     const int m = (int)(ws.pix_start[q + 1] - s0);
     float T;
@@ -2081,7 +2130,7 @@ inpc_status launch_scatter(const RP& P, const float* pos, const float* opacity, 
 // kept in the workspace for the backward).
 template <class FT>
 inpc_status bin_fragments(const RP& P, const float* pos, const float* opacity, const FT* feat, const RasterWs& ws,
-                          uint32_t cap_small, uint32_t cap_group, cudaStream_t s) {
+                          ClassCaps cap, cudaStream_t s) {
   INPC_CUDA(cudaMemsetAsync(ws.pix_count, 0, sizeof(uint32_t) * P.n_pix, s), "clear pixel counts");
   if (P.n > 0) {
     INPC_TRY(P.n >= (long long)device_sm_count() * 2048 ? (launch_count<512, 2>(P, pos, ws, s))
@@ -2089,9 +2138,7 @@ inpc_status bin_fragments(const RP& P, const float* pos, const float* opacity, c
   }
   INPC_TRY((scan::run<uint32_t, CountLoad, false>(CountLoad{ws.pix_count}, P.n_pix, ws.pix_start, ws.tops, s)));
   const long long nb = ceil_div(P.n_pix, scan::kBlock);
-  k_classify<<<(unsigned)ceil_div(P.n_pix, 256), 256, 0, s>>>(ws.pix_start, P.n_pix, ws.tops, nb, cap_small, cap_group,
-                                                               ws.heavy, ws.heavy_count, ws.large, ws.large_count,
-                                                               ws.pix_start, 4 * (cap_small / 2), ws.wide_count);
+  k_classify<<<(unsigned)ceil_div(P.n_pix, 256), 256, 0, s>>>(P.n_pix, nb, cap, ws);
   INPC_TRY(check_launch("k_classify"));
   if (P.n > 0) {
     INPC_TRY(launch_scatter<FT>(P, pos, opacity, feat, ws, s));
@@ -2102,7 +2149,7 @@ inpc_status bin_fragments(const RP& P, const float* pos, const float* opacity, c
 template <int V, int GA, class FT>
 inpc_status launch_fwd(const RP& P, const float* pos, const float* opacity, const FT* feat, const RasterWs& ws,
                        FT* image, float* T_final, int32_t* n_contrib, cudaStream_t s) {
-  INPC_TRY(bin_fragments(P, pos, opacity, feat, ws, 2 * GA, GA * kRegMax, s));
+  INPC_TRY(bin_fragments(P, pos, opacity, feat, ws, ClassCaps{2 * GA, 4 * GA, GA * kRegMax}, s));
   static SmemOnce f2;
   INPC_TRY(set_smem(k_blend_fwd_heavy<V, GA, FT>, HeavyBuf::bytes(), f2));
   INPC_TIMED("k_blend_fwd", s,
@@ -2116,6 +2163,10 @@ inpc_status launch_fwd(const RP& P, const float* pos, const float* opacity, cons
              k_blend_fwd_large<V, GA, FT, kRegMax><<<device_sm_count() * 3, kThreads, 0, s>>>(P, feat, ws, image,
                                                                                             T_final, n_contrib));
   INPC_TRY(check_launch("k_blend_fwd_large"));
+  INPC_TIMED("k_blend_fwd_warp", s,
+             k_blend_fwd_warp<V, GA, FT><<<device_sm_count() * 3, kThreads, 0, s>>>(P, feat, ws, image, T_final,
+                                                                                  n_contrib));
+  INPC_TRY(check_launch("k_blend_fwd_warp"));
   INPC_TIMED("k_blend_fwd_heavy", s,
              k_blend_fwd_heavy<V, GA, FT><<<device_sm_count() * 4, kThreads, HeavyBuf::bytes(), s>>>(
                  P, feat, ws, image, T_final, n_contrib));
@@ -2132,7 +2183,7 @@ inpc_status launch_blend_bwd(const RP& P, const FT* feat, const int32_t* n_contr
   INPC_CUDA(cudaMemsetAsync(ws.heavy_count, 0, 4 * sizeof(uint32_t), s), "clear class counts");
   INPC_TIMED("k_classify_bwd", s,
              k_classify_bwd<<<(unsigned)ceil_div(P.n_pix, 256), 256, 0, s>>>(
-                 n_contrib, ws.pix_start, P.n_pix, 2 * GA, GA * kRegMax, ws.heavy, ws.heavy_count, ws.large,
+                 n_contrib, ws.pix_start, P.n_pix, 2 * GA, kCandMax, ws.heavy, ws.heavy_count, ws.large,
                  ws.large_count));
   INPC_TRY(check_launch("k_classify_bwd"));
   INPC_TIMED("k_blend_bwd", s, k_blend_bwd<V, GA, FT><<<P.n_tiles, kThreads, 0, s>>>(P, feat, n_contrib, d_image, ws));
