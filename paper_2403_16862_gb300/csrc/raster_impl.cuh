@@ -41,6 +41,7 @@
 #include <climits>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "scan.cuh"
@@ -1068,28 +1069,39 @@ __device__ void blend_fwd_reg(const Group<GA>& G, const RP& P, const RasterWs& w
   }
 }
 
+}  // namespace
+}  // namespace inpc
+
+#include "raster_small.cuh"
+
+namespace inpc {
+namespace {
+
 // A tile's pixels in shared memory: bucket start, size (-1 outside the
 // image) and blended count of tile pixel i, loaded by thread i
-// (TW * TH <= kThreads), and the list of the pixels this kernel works on.
-// The CTA's groups take pixels from the list through a cursor, so a group
-// done with small buckets takes more and no warp waits on another's share.
+// (TW * TH <= kThreads), and the lists of the pixels this kernel works on:
+// list 0 for one lane group per pixel, and for 64 channels lists 1 and 2 of
+// at most 8 and 16 fragments (raster_small.cuh).  The CTA's groups take
+// pixels from the lists through cursors, so a group done with small buckets
+// takes more and no warp waits on another's share.
 struct TileSmem {
   uint32_t s0[kThreads];
   int m[kThreads];
   int nb[kThreads];
-  uint16_t list[kThreads];
-  int count, next;
+  uint16_t list[3][kThreads];
+  int count[3], next[3];
+  uint8_t src[kThreads];  // exchange space of the warps' sorts
 };
 
 // kBwd: the work pixels are those with 0 < blended count <= cap (else
 // 0 < bucket size <= cap).
-template <bool kBwd>
+template <bool kBwd, bool kSmall>
 __device__ __forceinline__ void load_tile(const RP& P, const RasterWs& ws, int tx, int ty,
                                           const int32_t* __restrict__ n_contrib, int cap, TileSmem& S) {
   const int i = threadIdx.x;
-  if (i == 0) {
-    S.count = 0;
-    S.next = 0;
+  if (i < 3) {
+    S.count[i] = 0;
+    S.next[i] = 0;
   }
   __syncthreads();
   if (i < P.TW * P.TH) {
@@ -1106,18 +1118,34 @@ __device__ __forceinline__ void load_tile(const RP& P, const RasterWs& ws, int t
     S.m[i] = m;
     S.nb[i] = nb;
     const int w = kBwd ? nb : m;
-    if (w > 0 && w <= cap) S.list[atomicAdd(&S.count, 1)] = (uint16_t)i;
+    if (w > 0 && w <= cap) {
+      const int which = !kSmall || w > 16 ? 0 : w <= 8 ? 1 : 2;
+      S.list[which][atomicAdd(&S.count[which], 1)] = (uint16_t)i;
+    }
   }
   __syncthreads();
 }
 
-// The next work pixel of the tile for this group, or -1.
+// The next work pixel of list 0 for this group, or -1.
 template <int GA>
 __device__ __forceinline__ int next_tile_pixel(const Group<GA>& G, TileSmem& S) {
   int k = 0;
-  if (G.lg == 0) k = atomicAdd(&S.next, 1);
+  if (G.lg == 0) k = atomicAdd(&S.next[0], 1);
   k = G.bcast(k, 0);
-  return k < S.count ? (int)S.list[k] : -1;
+  return k < S.count[0] ? (int)S.list[0][k] : -1;
+}
+
+// The next pixels of list `which` for the warp's 32 / LP lane groups: this
+// group's pixel, or -1; false when the list is done.
+template <int LP>
+__device__ __forceinline__ bool next_small_pixels(TileSmem& S, int which, int& j) {
+  const int lane = threadIdx.x & 31;
+  int k = 0;
+  if (lane == 0) k = atomicAdd(&S.next[which], 32 / LP);
+  k = __shfl_sync(0xffffffffu, k, 0);
+  const int mine = k + lane / LP;
+  j = mine < S.count[which] ? (int)S.list[which][mine] : -1;
+  return k < S.count[which];
 }
 
 __device__ __forceinline__ long long tile_pixel_index(const RP& P, int tx, int ty, int j) {
@@ -1157,7 +1185,8 @@ __global__ void __launch_bounds__(kThreads, 5) k_blend_fwd(RP P, const FT* __res
   const Group<GA> G;
   const int t = blockIdx.x;
   const int tx = t % P.tiles_x, ty = t / P.tiles_x;
-  load_tile<false>(P, ws, tx, ty, nullptr, 2 * GA, S);
+  constexpr bool kSmall = V == 2 && GA == 32;  // 64 channels
+  load_tile<false, kSmall>(P, ws, tx, ty, nullptr, 2 * GA, S);
   fill_empty<FT>(P, tx, ty, S, image, T_final, n_contrib);
   // the next pixel is taken before the current one is blended
   for (int j = next_tile_pixel(G, S); j >= 0;) {
@@ -1168,6 +1197,19 @@ __global__ void __launch_bounds__(kThreads, 5) k_blend_fwd(RP P, const FT* __res
     if (m <= GA) blend_fwd_reg<V, GA, FT, 1>(G, P, ws, s0, m, q, feat, image, T_final, n_contrib);
     else blend_fwd_reg<V, GA, FT, 2>(G, P, ws, s0, m, q, feat, image, T_final, n_contrib);
     j = jn;
+  }
+  if constexpr (kSmall) {
+    uint8_t* const src = S.src + (threadIdx.x & ~31);
+    const auto small = [&](auto lp, int which) {
+      constexpr int LP = decltype(lp)::value;
+      const Group<LP> L;
+      for (int j; next_small_pixels<LP>(S, which, j);)
+        blend_fwd_small<FT, LP>(L, P, ws, j < 0 ? 0u : S.s0[j], j < 0 ? 0 : S.m[j],
+                                j < 0 ? 0ll : tile_pixel_index(P, tx, ty, j), src + L.base_lane, feat, image, T_final,
+                                n_contrib);
+    };
+    small(std::integral_constant<int, 16>(), 2);
+    small(std::integral_constant<int, 8>(), 1);
   }
 }
 
@@ -1283,7 +1325,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_bwd(RP P, const FT* __res
   const Group<GA> G;
   const int t = blockIdx.x;
   const int tx = t % P.tiles_x, ty = t / P.tiles_x;
-  load_tile<true>(P, ws, tx, ty, n_contrib, 2 * GA, S);
+  constexpr bool kSmall = V == 2 && GA == 32;  // 64 channels
+  load_tile<true, kSmall>(P, ws, tx, ty, n_contrib, 2 * GA, S);
   // the next pixel is taken before the current one is revisited
   for (int j = next_tile_pixel(G, S); j >= 0;) {
     const int jn = next_tile_pixel(G, S);
@@ -1294,6 +1337,17 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_bwd(RP P, const FT* __res
     if (nb <= GA) blend_bwd_reg<V, GA, FT, 1>(G, P, ws, s0, m, nb, q, feat, d_image);
     else blend_bwd_reg<V, GA, FT, 2>(G, P, ws, s0, m, nb, q, feat, d_image);
     j = jn;
+  }
+  if constexpr (kSmall) {
+    const auto small = [&](auto lp, int which) {
+      constexpr int LP = decltype(lp)::value;
+      const Group<LP> L;
+      for (int j; next_small_pixels<LP>(S, which, j);)
+        blend_bwd_small<FT, LP>(L, P, ws, j < 0 ? 0u : S.s0[j], j < 0 ? 0 : S.m[j], j < 0 ? 0 : S.nb[j],
+                                j < 0 ? 0ll : tile_pixel_index(P, tx, ty, j), feat, d_image);
+    };
+    small(std::integral_constant<int, 16>(), 2);
+    small(std::integral_constant<int, 8>(), 1);
   }
 }
 
