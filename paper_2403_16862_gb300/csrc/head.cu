@@ -36,15 +36,19 @@ ShConsts make_consts(const inpc_camera& cam) {
 
 // The direction is formed in FP64: x - o cancels for points near a
 // coordinate plane through the camera, and FP32 would lose the small
-// component's relative accuracy there.
+// component's relative accuracy there.  FP64 runs at a few lanes per SM and
+// clock, so the three divisions and the square root are one reciprocal
+// square root and three products (about 23 FP64 operations instead of 75;
+// the results are rounded to FP32 either way).
 __device__ __forceinline__ void sh9(const ShConsts& k, const float* p, float Y[9]) {
   const double vx = (double)p[0] - k.o[0], vy = (double)p[1] - k.o[1], vz = (double)p[2] - k.o[2];
-  const double len = sqrt(vx * vx + vy * vy + vz * vz);
+  const double len2 = vx * vx + vy * vy + vz * vz;
   float x = 0.f, y = 0.f, z = 1.f;
-  if (len > 0.0) {
-    x = (float)(vx / len);
-    y = (float)(vy / len);
-    z = (float)(vz / len);
+  if (len2 > 0.0) {
+    const double inv = rsqrt(len2);
+    x = (float)(vx * inv);
+    y = (float)(vy * inv);
+    z = (float)(vz * inv);
   }
   Y[0] = k.c0;
   Y[1] = k.c1 * y;
@@ -77,48 +81,130 @@ __global__ void k_contract(const float* __restrict__ pos, int64_t n, float cx, f
   }
 }
 
-template <class HT>
-__global__ void k_sh_head_fwd(ShConsts k, const float* __restrict__ pos, const HT* __restrict__ h, int64_t n, int F,
-                              float* __restrict__ alpha, float* __restrict__ color) {
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
+// Four features from element e of a row.
+__device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
+  const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16),
+                     __uint_as_float(r.y & 0xFFFF0000u));
+}
+
+constexpr int kHeadThreads = 128;
+constexpr int kHeadFeats = 37;   // opacity and 36 SH features
+constexpr int kHeadStride = 41;  // shared-memory row of a point (odd: the lanes' rows start in different banks)
+
+// A warp takes 32 consecutive points: it reads their rows' first 37 (kVec:
+// 40, 4 at a time) features side by side into shared memory, then each lane
+// works on its own point.  (One thread per point reading its row directly
+// touched 32 lines per load: 500k points, 64 features, 78 us.)
+template <class HT, bool kVec>
+__global__ void __launch_bounds__(kHeadThreads) k_sh_head_fwd(ShConsts k, const float* __restrict__ pos,
+                                                              const HT* __restrict__ h, int64_t n, int F,
+                                                              float* __restrict__ alpha, float* __restrict__ color) {
+  __shared__ float rows_s[kHeadThreads / 32][32 * kHeadStride];
+  const int lane = threadIdx.x & 31;
+  float* rows = rows_s[threadIdx.x >> 5];
+  const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; 32 * b < n; b += n_warps) {
+    const int64_t p0 = 32 * b;
+    const int np = (int)min((int64_t)32, n - p0);
+    __syncwarp();
+    if (kVec) {
+#pragma unroll
+      for (int i = 0; i < 10; ++i) {
+        const int pt = (i * 32 + lane) / 10, e = 4 * ((i * 32 + lane) % 10);
+        if (pt < np) {
+          const float4 v = ld4(h + (p0 + pt) * F + e);
+          float* o = rows + pt * kHeadStride + e;
+          o[0] = v.x;
+          o[1] = v.y;
+          o[2] = v.z;
+          o[3] = v.w;
+        }
+      }
+    } else {
+      for (int i = lane; i < np * kHeadFeats; i += 32)
+        rows[i / kHeadFeats * kHeadStride + i % kHeadFeats] = ldf(h + (p0 + i / kHeadFeats) * F + i % kHeadFeats);
+    }
+    __syncwarp();
+    if (lane >= np) continue;
+    const int64_t p = p0 + lane;
     float Y[9];
     sh9(k, pos + 3 * p, Y);
-    const HT* row = h + (int64_t)F * p;
-    alpha[p] = -expm1f(-expf(ldf(row)));
+    const float* row = rows + lane * kHeadStride;
+    alpha[p] = -expm1f(-expf(row[0]));
     float c[4];
 #pragma unroll
     for (int ch = 0; ch < 4; ++ch) {
       float s = 0.f;
 #pragma unroll
-      for (int b = 0; b < 9; ++b) s = fmaf(Y[b], ldf(row + 1 + 9 * ch + b), s);
+      for (int q = 0; q < 9; ++q) s = fmaf(Y[q], row[1 + 9 * ch + q], s);
       c[ch] = s;
     }
     reinterpret_cast<float4*>(color)[p] = make_float4(c[0], c[1], c[2], c[3]);
   }
 }
 
-template <class HT>
-__global__ void k_sh_head_bwd(ShConsts k, const float* __restrict__ pos, const HT* __restrict__ h, int64_t n, int F,
-                              const float* __restrict__ d_alpha, const float* __restrict__ d_color,
-                              float* __restrict__ dh) {
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    float Y[9];
-    sh9(k, pos + 3 * p, Y);
-    float* out = dh + (int64_t)F * p;
-    const float e = expf(ldf(h + (int64_t)F * p));
-    out[0] = d_alpha[p] * (e * expf(-e));
-    const float4 g = reinterpret_cast<const float4*>(d_color)[p];
-    const float gc[4] = {g.x, g.y, g.z, g.w};
+// The derivative: each lane forms one point's basis and color gradient into
+// shared memory, then the warp writes the 32 rows of dh side by side (kVec:
+// 4 values per lane).  (Each thread writing its own row: 500k points, 64
+// features, 178 us.)
+template <class HT, bool kVec>
+__global__ void __launch_bounds__(kHeadThreads) k_sh_head_bwd(ShConsts k, const float* __restrict__ pos,
+                                                              const HT* __restrict__ h, int64_t n, int F,
+                                                              const float* __restrict__ d_alpha,
+                                                              const float* __restrict__ d_color,
+                                                              float* __restrict__ dh) {
+  constexpr int kRec = 15;  // basis (9), color gradient (4), opacity path
+  __shared__ float rec_s[kHeadThreads / 32][32 * kRec];
+  const int lane = threadIdx.x & 31;
+  float* rec = rec_s[threadIdx.x >> 5];
+  const auto value = [&](const float* r, int f) {
+    if (f == 0) return r[13];
+    if (f >= kHeadFeats) return 0.f;
+    return r[(f - 1) % 9] * r[9 + (f - 1) / 9];
+  };
+  const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; 32 * b < n; b += n_warps) {
+    const int64_t p0 = 32 * b;
+    const int np = (int)min((int64_t)32, n - p0);
+    __syncwarp();
+    if (lane < np) {
+      const int64_t p = p0 + lane;
+      float Y[9];
+      sh9(k, pos + 3 * p, Y);
+      float* r = rec + lane * kRec;
 #pragma unroll
-    for (int ch = 0; ch < 4; ++ch)
-#pragma unroll
-      for (int b = 0; b < 9; ++b) out[1 + 9 * ch + b] = Y[b] * gc[ch];
-    for (int f = 37; f < F; ++f) out[f] = 0.f;
+      for (int q = 0; q < 9; ++q) r[q] = Y[q];
+      const float4 g = reinterpret_cast<const float4*>(d_color)[p];
+      r[9] = g.x;
+      r[10] = g.y;
+      r[11] = g.z;
+      r[12] = g.w;
+      const float e = expf(ldf(h + F * p));
+      r[13] = d_alpha[p] * (e * expf(-e));
+    }
+    __syncwarp();
+    float* out = dh + p0 * F;
+    if (kVec) {
+      const int parts = F / 4;
+      for (int i = lane; i < np * parts; i += 32) {
+        const float* r = rec + i / parts * kRec;
+        const int f = 4 * (i % parts);
+        reinterpret_cast<float4*>(out)[i] = make_float4(value(r, f), value(r, f + 1), value(r, f + 2), value(r, f + 3));
+      }
+    } else {
+      for (int i = lane; i < np * F; i += 32) out[i] = value(rec + i / F * kRec, i % F);
+    }
   }
 }
 
 unsigned grid_for_points(int64_t n) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), (int64_t)device_sm_count() * 16));
+}
+
+unsigned grid_for_warps(int64_t n) {
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, kHeadThreads), (int64_t)device_sm_count() * 16));
 }
 
 inpc_status check_head(const inpc_camera* cam, const float* pos, const void* h, int32_t dtype, int64_t n, int32_t F) {
@@ -156,12 +242,15 @@ extern "C" inpc_status inpc_sh_head_fwd(const inpc_camera* cam, const float* pos
   if (!alpha_out || !color_out || !aligned(color_out, 16)) return fail(INPC_ERR_INVALID_ARG, "bad output pointer");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const ShConsts k = make_consts(*cam);
-  if (h_dtype == INPC_F32)
-    k_sh_head_fwd<float><<<grid_for_points(n), 256, 0, s>>>(k, pos, static_cast<const float*>(h), n, n_channels,
-                                                             alpha_out, color_out);
-  else
-    k_sh_head_fwd<__nv_bfloat16><<<grid_for_points(n), 256, 0, s>>>(k, pos, static_cast<const __nv_bfloat16*>(h), n,
-                                                                     n_channels, alpha_out, color_out);
+  // rows of 40 or more features whose 4-element groups are aligned
+  const bool vec = n_channels % 4 == 0 && n_channels >= 40 && aligned(h, h_dtype == INPC_F32 ? 16 : 8);
+  const auto run = [&](auto kernel, auto* rows) {
+    kernel<<<grid_for_warps(n), kHeadThreads, 0, s>>>(k, pos, rows, n, n_channels, alpha_out, color_out);
+  };
+  const float* hf = static_cast<const float*>(h);
+  const __nv_bfloat16* hb = static_cast<const __nv_bfloat16*>(h);
+  if (h_dtype == INPC_F32) vec ? run(k_sh_head_fwd<float, true>, hf) : run(k_sh_head_fwd<float, false>, hf);
+  else vec ? run(k_sh_head_fwd<__nv_bfloat16, true>, hb) : run(k_sh_head_fwd<__nv_bfloat16, false>, hb);
   return check_launch("k_sh_head_fwd");
 }
 
@@ -174,11 +263,13 @@ extern "C" inpc_status inpc_sh_head_bwd(const inpc_camera* cam, const float* pos
   if (!d_alpha || !d_color || !dh_out || !aligned(d_color, 16)) return fail(INPC_ERR_INVALID_ARG, "bad pointer");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const ShConsts k = make_consts(*cam);
-  if (h_dtype == INPC_F32)
-    k_sh_head_bwd<float><<<grid_for_points(n), 256, 0, s>>>(k, pos, static_cast<const float*>(h), n, n_channels,
-                                                             d_alpha, d_color, dh_out);
-  else
-    k_sh_head_bwd<__nv_bfloat16><<<grid_for_points(n), 256, 0, s>>>(k, pos, static_cast<const __nv_bfloat16*>(h), n,
-                                                                     n_channels, d_alpha, d_color, dh_out);
+  const bool vec = n_channels % 4 == 0 && aligned(dh_out, 16);
+  const auto run = [&](auto kernel, auto* rows) {
+    kernel<<<grid_for_warps(n), kHeadThreads, 0, s>>>(k, pos, rows, n, n_channels, d_alpha, d_color, dh_out);
+  };
+  const float* hf = static_cast<const float*>(h);
+  const __nv_bfloat16* hb = static_cast<const __nv_bfloat16*>(h);
+  if (h_dtype == INPC_F32) vec ? run(k_sh_head_bwd<float, true>, hf) : run(k_sh_head_bwd<float, false>, hf);
+  else vec ? run(k_sh_head_bwd<__nv_bfloat16, true>, hb) : run(k_sh_head_bwd<__nv_bfloat16, false>, hb);
   return check_launch("k_sh_head_bwd");
 }
