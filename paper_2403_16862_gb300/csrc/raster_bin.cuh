@@ -13,11 +13,21 @@
 // goes to its global counter directly.
 //
 // With one global atomic per fragment the counting pass ran at the L2's
-// atomic rate (253M atomics in 1.29 ms = 196G/s for 67M points), and the
-// scattering pass waited on returning atomics and left most sectors of the
-// buckets partly written.  The scattering pass now also sorts a chunk's
-// fragments by pixel in shared memory, so that a bucket receives runs of
-// consecutive keys.
+// atomic rate (253M atomics in 1.29 ms = 196G/s for 67M points; 0.58 ms with
+// the window, now bound by issue at 69 % of the slots), and the scattering
+// pass waited on returning atomics and left most sectors of the buckets partly
+// written.  The scattering pass also sorts a chunk's fragments by pixel in
+// shared memory, so that a bucket receives runs of consecutive keys: without
+// the sort the stores alone, a sector each, take 5.0 ms for 67M points.
+//
+// Scattering 67M points (1280 x 832, BF16 rows): 5.44 ms direct, 3.86 ms with
+// a list of the counters in use, 3.13 ms with a footprint's four counters in
+// flight together and the window read as a whole in place of the list; 16M
+// 1.44, 1.12 and 0.89 ms; 4M (FP32) 367, 346 and 272 us.  What bounds it now
+// is the memory's handling of partly written sectors (16M points: 1.07 GB
+// written, 2.56 GB read of which 0.74 GB are inputs, at 4.05 TB/s).  Larger
+// chunks, more resident warps and streaming hints on the inputs measured the
+// same or slower.
 #pragma once
 
 namespace inpc {
@@ -32,13 +42,6 @@ constexpr int kWinCountBits = 14;
 constexpr uint32_t kWinCountMask = (1u << kWinCountBits) - 1;
 constexpr uint32_t kWinFree = 0xFFFFFFFFu;
 constexpr uint32_t kNoRank = 0xFFFFu;
-
-// The window: words, and the list of the counters in use.
-struct BinWindow {
-  uint32_t* word;   // [kWinSlots]
-  uint16_t* list;   // [min(kWinSlots, fragments of a chunk)]
-  int* n_list;
-};
 
 // Counter of pixel (x, y); the rows are skewed so that a few pixels of
 // several rows spread over the shared-memory banks.
@@ -58,48 +61,73 @@ __device__ __forceinline__ uint32_t win_pixel(int slot, uint32_t w, int W) {
   return (uint32_t)(y * W + x);
 }
 
-// Counts a fragment of pixel (x, y): its rank among the chunk's fragments of
-// that pixel, or kNoRank when another pixel holds the counter.
-__device__ __forceinline__ uint32_t win_take(const BinWindow& B, int x, int y) {
-  const int slot = win_slot(x, y);
-  const uint32_t fresh = win_tag(x, y) << kWinCountBits;
-  uint32_t w = *(volatile uint32_t*)(B.word + slot);
-  if (w == kWinFree) {
-    w = atomicCAS(B.word + slot, kWinFree, fresh);
-    if (w == kWinFree) {
-      B.list[atomicAdd(B.n_list, 1)] = (uint16_t)slot;
-      w = fresh;
+// Counts the (up to four) fragments of a footprint: the rank of each among the
+// chunk's fragments of its pixel, or kNoRank when another pixel holds the
+// counter (or the corner is off the image), two ranks to a word.  A footprint's
+// corners have four different counters, so the reads, the claims and the
+// additions of the four go out together.
+__device__ __forceinline__ void win_take(const RP& P, uint32_t* word, const Footprint& f, uint32_t (&rank)[2]) {
+  int slot[4];
+  uint32_t fresh[4], w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int x = f.i0 + (k & 1), y = f.j0 + (k >> 1);
+    slot[k] = win_slot(x, y);
+    fresh[k] = win_tag(x, y) << kWinCountBits;
+    w[k] = *(volatile uint32_t*)(word + slot[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (corner_pixel(P, f, k) < 0) {
+      w[k] = ~fresh[k];  // no counter of this tag
+    } else if (w[k] == kWinFree) {
+      w[k] = atomicCAS(word + slot[k], kWinFree, fresh[k]);
+      if (w[k] == kWinFree) w[k] = fresh[k];
     }
   }
-  if ((w ^ fresh) >> kWinCountBits) return kNoRank;
-  return atomicAdd(B.word + slot, 1u) & kWinCountMask;
+  uint32_t r[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    r[k] = (w[k] ^ fresh[k]) >> kWinCountBits ? kNoRank : atomicAdd(word + slot[k], 1u) & kWinCountMask;
+  rank[0] = r[0] | (r[1] << 16);
+  rank[1] = r[2] | (r[3] << 16);
+}
+
+__device__ __forceinline__ uint32_t rank_of(const uint32_t (&rank)[2], int k) {
+  return (rank[k >> 1] >> (16 * (k & 1))) & 0xffffu;
 }
 
 // A CTA of kT threads bins chunks of kT * kPP consecutive points.
 template <int kT, int kPP>
-struct BinSmem {
+struct BinShape {
   static constexpr int kPoints = kT * kPP;
-  static constexpr int kFrags = 4 * kPoints;
-  static constexpr int kList = kFrags < kWinSlots ? kFrags : kWinSlots;
-  static_assert(kFrags <= (int)kWinCountMask, "a chunk's count fits its field");
-  uint32_t word[kWinSlots];
-  uint16_t list[kList];
-  int n_list[2];   // alternate over the chunks
-  int n_sorted[2];
+  static_assert(4 * kPoints <= (int)kWinCountMask, "a chunk's count fits its field");
+  static constexpr int kScan = kWinSlots / (4 * kT);  // 16-byte groups of counters per thread
+  static_assert(kScan * 4 * kT == kWinSlots, "the threads share the window evenly");
 };
 
+// What the counting pass leaves for the choice of the scattering pass: the
+// fragments in the windows of a few CTAs' first chunks, and the counters they
+// took.  An unordered cloud has hardly more fragments than counters; there
+// the window is only work (16M points in no order at 1280 x 832: 2.74 ms with
+// it, 2.36 ms without; grouped by leaf 0.89 and 1.44 ms).
+struct WinSample {
+  uint32_t used, frags;
+};
+constexpr int kSampleEvery = 16;  // CTAs per sampled one
+
+__device__ __forceinline__ bool window_wanted(const WinSample* s) { return 4u * s->frags >= 5u * s->used; }
+
+// sample: null where the scattering pass has no use for it.
 template <int kT, int kPP>
 __global__ void __launch_bounds__(kT) k_pix_count(RP P, const float* __restrict__ pos,
-                                                  uint32_t* __restrict__ pix_count) {
-  using Smem = BinSmem<kT, kPP>;
-  __shared__ Smem S;
-  for (int i = threadIdx.x; i < kWinSlots; i += kT) S.word[i] = kWinFree;
-  if (threadIdx.x < 2) S.n_list[threadIdx.x] = 0;
+                                                  uint32_t* __restrict__ pix_count, WinSample* sample) {
+  using Shape = BinShape<kT, kPP>;
+  __shared__ __align__(16) uint32_t word[kWinSlots];
+  for (int i = threadIdx.x; i < kWinSlots; i += kT) word[i] = kWinFree;
   __syncthreads();
   const int n = (int)P.n;  // <= 2^28
-  int turn = 0;
-  for (int c0 = blockIdx.x * Smem::kPoints; c0 < n; c0 += gridDim.x * Smem::kPoints, turn ^= 1) {
-    const BinWindow B{S.word, S.list, &S.n_list[turn]};
+  for (int c0 = blockIdx.x * Shape::kPoints; c0 < n; c0 += gridDim.x * Shape::kPoints) {
     float xyz[kPP][3];
 #pragma unroll
     for (int u = 0; u < kPP; ++u) {
@@ -111,52 +139,72 @@ __global__ void __launch_bounds__(kT) k_pix_count(RP P, const float* __restrict_
     for (int u = 0; u < kPP; ++u) {
       Splat s;
       if (c0 + u * kT + (int)threadIdx.x >= n || !splat_xyz(P, xyz[u][0], xyz[u][1], xyz[u][2], s)) continue;
+      uint32_t rank[2];
+      win_take(P, word, s.f, rank);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int q = corner_pixel(P, s.f, k);
-        if (q >= 0 && win_take(B, s.f.i0 + (k & 1), s.f.j0 + (k >> 1)) == kNoRank) atomicAdd(pix_count + q, 1u);
+        if (q >= 0 && rank_of(rank, k) == kNoRank) atomicAdd(pix_count + q, 1u);
       }
     }
     __syncthreads();
-    const int m = S.n_list[turn];
-    if (threadIdx.x == 0) S.n_list[turn ^ 1] = 0;
-    for (int e = threadIdx.x; e < m; e += kT) {
-      const int slot = S.list[e];
-      const uint32_t w = S.word[slot];
-      S.word[slot] = kWinFree;
-      atomicAdd(pix_count + win_pixel(slot, w, P.cam.W), w & kWinCountMask);
+    if (sample && blockIdx.x % kSampleEvery == 0 && c0 == (int)blockIdx.x * Shape::kPoints) {
+      unsigned used = 0, frags = 0;
+      for (int i = threadIdx.x; i < kWinSlots; i += kT) {
+        if (word[i] == kWinFree) continue;
+        ++used;
+        frags += word[i] & kWinCountMask;
+      }
+      used = __reduce_add_sync(0xffffffffu, used);
+      frags = __reduce_add_sync(0xffffffffu, frags);
+      if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&sample->used, used);
+        atomicAdd(&sample->frags, frags);
+      }
+      __syncthreads();
+    }
+    // the counters go to the pixels and are free again
+#pragma unroll
+    for (int i = 0; i < Shape::kScan; ++i) {
+      const int slot = 4 * (i * kT + (int)threadIdx.x);
+      const uint4 w4 = *reinterpret_cast<const uint4*>(word + slot);
+      if ((w4.x & w4.y & w4.z & w4.w) == kWinFree) continue;
+      const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (w[j] != kWinFree) atomicAdd(pix_count + win_pixel(slot + j, w[j], P.cam.W), w[j] & kWinCountMask);
+      *reinterpret_cast<uint4*>(word + slot) = make_uint4(kWinFree, kWinFree, kWinFree, kWinFree);
     }
     __syncthreads();
   }
 }
 
-// Dynamic shared memory of the scattering pass: the window, then per counter
-// the global slot of the chunk's first fragment, then the chunk's fragments
-// sorted by pixel (key, alpha, global slot).
+// Dynamic shared memory of the scattering pass: the chunk's fragments sorted
+// by pixel (key, alpha, bucket slot), the window, and per counter the bucket
+// slot of the chunk's first fragment.
 template <int kT, int kPP>
 struct ScatterSmem {
-  using Bin = BinSmem<kT, kPP>;
-  unsigned long long key[Bin::kFrags];
-  float alpha[Bin::kFrags];
-  uint32_t dst[Bin::kFrags];
+  static constexpr int kFrags = 4 * kT * kPP;
+  unsigned long long key[kFrags];
+  float alpha[kFrags];
+  uint32_t dst[kFrags];
+  uint32_t word[kWinSlots];
   uint32_t base[kWinSlots];
-  Bin bin;
+  int n_sorted[2];  // alternate over the chunks
 };
 
 template <int kT, int kPP, class FT>
 __global__ void __launch_bounds__(kT, 1024 / kT) k_pix_scatter(RP P, const float* __restrict__ pos,
-                                                               const float* __restrict__ opacity,
-                                                               const FT* __restrict__ feat, RasterWs ws) {
-  using Smem = ScatterSmem<kT, kPP>;
-  constexpr int kPoints = Smem::Bin::kPoints;
+                                                           const float* __restrict__ opacity,
+                                                           const FT* __restrict__ feat, RasterWs ws) {
+  using Shape = BinShape<kT, kPP>;
+  constexpr int kPoints = Shape::kPoints;
+  if (!window_wanted(ws.sample)) return;
   extern __shared__ __align__(16) unsigned char dyn[];
-  Smem& S = *reinterpret_cast<Smem*>(dyn);
+  ScatterSmem<kT, kPP>& S = *reinterpret_cast<ScatterSmem<kT, kPP>*>(dyn);
   const int lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < kWinSlots; i += kT) S.bin.word[i] = kWinFree;
-  if (threadIdx.x < 2) {
-    S.bin.n_list[threadIdx.x] = 0;
-    S.bin.n_sorted[threadIdx.x] = 0;
-  }
+  for (int i = threadIdx.x; i < kWinSlots; i += kT) S.word[i] = kWinFree;
+  if (threadIdx.x < 2) S.n_sorted[threadIdx.x] = 0;
   __syncthreads();
   const int n = (int)P.n;  // <= 2^28
   int turn = 0;
@@ -174,61 +222,60 @@ __global__ void __launch_bounds__(kT, 1024 / kT) k_pix_scatter(RP P, const float
   };
   load((long long)blockIdx.x * kPoints);
   for (int c0 = blockIdx.x * kPoints; c0 < n; c0 += gridDim.x * kPoints, turn ^= 1) {
-    const BinWindow B{S.bin.word, S.bin.list, &S.bin.n_list[turn]};
-    float xyz[kPP][3], av[kPP];
-#pragma unroll
-    for (int u = 0; u < kPP; ++u) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a) xyz[u][a] = next[u][a];
-      av[u] = next[u][3];
-    }
     // the chunk's fragments: their rank within their pixel
     Splat s[kPP];
+    float av[kPP];
     uint32_t rank[kPP][2];
     unsigned ok = 0;
 #pragma unroll
     for (int u = 0; u < kPP; ++u) {
-      rank[u][0] = rank[u][1] = 0u;
-      const int id = c0 + u * kT + (int)threadIdx.x;
-      const bool in = id < n && splat_xyz(P, xyz[u][0], xyz[u][1], xyz[u][2], s[u]);
-      if (in) {
+      av[u] = next[u][3];
+      if (c0 + u * kT + (int)threadIdx.x < n && splat_xyz(P, next[u][0], next[u][1], next[u][2], s[u])) {
         ok |= 1u << u;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int q = corner_pixel(P, s[u].f, k);
-          if (q >= 0) rank[u][k >> 1] |= win_take(B, s[u].f.i0 + (k & 1), s[u].f.j0 + (k >> 1)) << (16 * (k & 1));
-        }
+        win_take(P, S.word, s[u].f, rank[u]);
       }
     }
     __syncthreads();
-    // one global atomic per pixel in use: the bucket slots of its fragments
-    // (the counts run down from the bucket size, so the buckets fill back to
-    // front) and their place in the sorted chunk
-    const int m = *B.n_list;
     load(c0 + (long long)gridDim.x * kPoints);
-    for (int e0 = (int)threadIdx.x - lane; e0 < m; e0 += kT) {
-      const int e = e0 + lane;
-      int slot = 0;
-      uint32_t c = 0, first = 0;
-      if (e < m) {
-        slot = S.bin.list[e];
-        const uint32_t w = S.bin.word[slot];
-        const uint32_t q = win_pixel(slot, w, P.cam.W);
-        c = w & kWinCountMask;
-        first = __ldg(ws.pix_start + q) + atomicSub(ws.pix_count + q, c) - c;
+    // one global atomic per pixel in use gives the bucket slots of its
+    // fragments (the counts run down from the bucket size, so the buckets
+    // fill back to front) and its place in the sorted chunk replaces the
+    // counter.  The window is read as a whole: a thread's few counters are
+    // all in flight together.
+#pragma unroll
+    for (int i = 0; i < Shape::kScan; ++i) {
+      const int slot = 4 * (i * kT + (int)threadIdx.x);
+      const uint4 w4 = *reinterpret_cast<const uint4*>(S.word + slot);
+      const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+      const bool used = (w4.x & w4.y & w4.z & w4.w) != kWinFree;
+      if (!__any_sync(0xffffffffu, used)) continue;
+      uint32_t first[4] = {0, 0, 0, 0}, c[4], incl = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        c[j] = w[j] != kWinFree ? w[j] & kWinCountMask : 0u;
+        if (c[j]) {
+          const uint32_t q = win_pixel(slot + j, w[j], P.cam.W);
+          first[j] = __ldg(ws.pix_start + q) + atomicSub(ws.pix_count + q, c[j]) - c[j];
+        }
+        incl += c[j];
       }
-      uint32_t incl = c;
+      const uint32_t mine = incl;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += t;
       }
       int at = 0;
-      if (lane == 31) at = atomicAdd(&S.bin.n_sorted[turn], (int)incl);
-      at = __shfl_sync(0xffffffffu, at, 31);
-      if (e < m) {
-        S.bin.word[slot] = (uint32_t)at + incl - c;
-        S.base[slot] = first;
+      if (lane == 31) at = atomicAdd(&S.n_sorted[turn], (int)incl);
+      at = __shfl_sync(0xffffffffu, at, 31) + (int)(incl - mine);
+      uint4 place;
+      place.x = at;
+      place.y = place.x + c[0];
+      place.z = place.y + c[1];
+      place.w = place.z + c[2];
+      if (used) {
+        *reinterpret_cast<uint4*>(S.word + slot) = place;
+        *reinterpret_cast<uint4*>(S.base + slot) = make_uint4(first[0], first[1], first[2], first[3]);
       }
     }
     __syncthreads();
@@ -249,17 +296,17 @@ __global__ void __launch_bounds__(kT, 1024 / kT) k_pix_scatter(RP P, const float
         for (int k = 0; k < 4; ++k) {
           const int q = corner_pixel(P, s[u].f, k);
           to[k] = 0;
-          if (q >= 0 && ((rank[u][k >> 1] >> (16 * (k & 1))) & 0xffffu) == kNoRank)
+          if (q >= 0 && rank_of(rank[u], k) == kNoRank)
             to[k] = __ldg(ws.pix_start + q) + atomicSub(ws.pix_count + q, 1u) - 1u;
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           if (corner_pixel(P, s[u].f, k) < 0) continue;
           const float a = fminf(__fmul_rn(ah, corner_weight(s[u].f, k & 1, k >> 1)), P.alpha_max);
-          const uint32_t r = (rank[u][k >> 1] >> (16 * (k & 1))) & 0xffffu;
+          const uint32_t r = rank_of(rank[u], k);
           if (r != kNoRank) {
             const int slot = win_slot(s[u].f.i0 + (k & 1), s[u].f.j0 + (k >> 1));
-            const uint32_t at = S.bin.word[slot] + r;
+            const uint32_t at = S.word[slot] + r;
             S.key[at] = key;
             S.alpha[at] = a;
             S.dst[at] = S.base[slot] + r;
@@ -275,27 +322,26 @@ __global__ void __launch_bounds__(kT, 1024 / kT) k_pix_scatter(RP P, const float
       }
     }
     __syncthreads();
-    const int total = S.bin.n_sorted[turn];
+    const int total = S.n_sorted[turn];
+    if (threadIdx.x == 0) S.n_sorted[turn ^ 1] = 0;
+#pragma unroll
+    for (int i = 0; i < Shape::kScan; ++i)
+      *reinterpret_cast<uint4*>(S.word + 4 * (i * kT + (int)threadIdx.x)) =
+          make_uint4(kWinFree, kWinFree, kWinFree, kWinFree);
     for (int j = threadIdx.x; j < total; j += kT) {
       const uint32_t to = S.dst[j];
       ws.keys[to] = S.key[j];
       ws.alpha[to] = S.alpha[j];
     }
-    for (int e = threadIdx.x; e < m; e += kT) S.bin.word[S.bin.list[e]] = kWinFree;
-    if (threadIdx.x == 0) {
-      S.bin.n_list[turn ^ 1] = 0;
-      S.bin.n_sorted[turn ^ 1] = 0;
-    }
     __syncthreads();
   }
 }
 
-// The scattering pass without the window, for clouds with few fragments per
-// pixel: one returning atomic per run of equal pixels over consecutive lanes.
-// A run of equal pixels over
-// consecutive lanes is found with one shuffle and one ballot (its start is a
-// lane whose pixel differs from the previous lane's), and its first lane
-// updates the counter for the whole run.
+// The scattering pass without the window, for small or unordered clouds (with
+// a sample, only where that does not ask for the window): one returning atomic
+// per run of equal pixels over consecutive lanes.  A run is found with one
+// shuffle and one ballot (its start is a lane whose pixel differs from the
+// previous lane's), and its first lane updates the counter for the whole run.
 struct LaneRun {
   int start;  // first lane of this lane's run
   int len;    // lanes in the run (valid in the first lane)
@@ -320,7 +366,9 @@ __global__ void __launch_bounds__(256) k_pix_scatter_direct(RP P, const float* _
                                                      uint32_t* __restrict__ pix_count,
                                                      unsigned long long* __restrict__ keys,
                                                      float* __restrict__ alpha, uint32_t* __restrict__ porg,
-                                                     float* __restrict__ pexp) {
+                                                     float* __restrict__ pexp,
+                                                     const WinSample* __restrict__ sample) {
+  if (sample && window_wanted(sample)) return;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int n = (int)P.n;  // <= 2^28

@@ -78,6 +78,8 @@ struct RP {
   unsigned long long idm;   // (1 << idb) - 1
 };
 
+struct WinSample;
+
 struct RasterWs {
   uint32_t* status;
   uint32_t* heavy_count;     // header word 1
@@ -89,6 +91,7 @@ struct RasterWs {
   uint32_t* select_count;    // header word 7: pixels with a selection by one warp (the front of mid)
   uint32_t* warp_count;      // header word 8: pixels with a whole bucket for one warp (the back of mid)
   uint32_t* warp_next;       // header word 9: the cursor over both
+  WinSample* sample;         // header words 10, 11: what the counting pass leaves for the scattering pass
   uint32_t* pix_count;       // [n_pix]
   uint32_t* pix_start;       // [n_pix + 1]
   uint32_t* tops;            // prefix-sum block totals
@@ -122,6 +125,7 @@ RasterWs carve(void* base, long long n_pix, long long n) {
   w.select_count = base ? reinterpret_cast<uint32_t*>(base) + 7 : nullptr;
   w.warp_count = base ? reinterpret_cast<uint32_t*>(base) + 8 : nullptr;
   w.warp_next = base ? reinterpret_cast<uint32_t*>(base) + 9 : nullptr;
+  w.sample = base ? reinterpret_cast<WinSample*>(reinterpret_cast<uint32_t*>(base) + 10) : nullptr;
   const long long nf = std::max<long long>(4 * n, 1);
   w.pix_count = c.take<uint32_t>(n_pix);
   w.pix_start = c.take<uint32_t>(n_pix + 1);
@@ -2147,36 +2151,44 @@ inpc_status set_smem(K kernel, size_t bytes, SmemOnce& once) {
 
 // Counting pass: chunks of kT kPP points.
 template <int kT, int kPP>
-inpc_status launch_count(const RP& P, const float* pos, const RasterWs& ws, cudaStream_t s) {
+inpc_status launch_count(const RP& P, const float* pos, const RasterWs& ws, WinSample* sample, cudaStream_t s) {
   const long long chunks = ceil_div(P.n, kT * kPP), resident = (long long)device_sm_count() * (2048 / kT);
   INPC_TIMED("k_pix_count", s,
-             k_pix_count<kT, kPP><<<(unsigned)std::min(chunks, resident), kT, 0, s>>>(P, pos, ws.pix_count));
+             k_pix_count<kT, kPP><<<(unsigned)std::min(chunks, resident), kT, 0, s>>>(P, pos, ws.pix_count, sample));
   return check_launch("k_pix_count");
 }
 
-// The window pays in the scattering pass where a chunk's pixels get several
-// fragments each and the chunks (1,024 points; two CTAs of 512 threads per
-// SM) fill the GPU several times over.  Measured, window against direct: 252
-// fragments a pixel (67M points) 3.74 and 5.68 ms, 16 (4M) 346 and 382 us, 15
-// (1M) 78 and 66 us, 4 (1M) 138 and 81 us.
+// The scattering pass's window pays where its chunks (1,024 points; two CTAs
+// of 512 threads per SM) fill the GPU several times over and the points come
+// grouped, which the counting pass finds out.  Measured on leaf-ordered
+// clouds, window against direct: 2M points on 641 x 417 pixels 108 and 132 us,
+// on 1280 x 832 139 and 168, on 3840 x 2160 191 and 205; 1.4M on 1000 x 700
+// 102 and 101 us; 1M on 1280 x 832 81 and 76 us; 262,144 on 320 x 240 18 and
+// 15 us.
+constexpr int kScatterT = 512, kScatterPP = 2;
+
+long long scatter_ctas() { return (long long)device_sm_count() * 2; }
+
+bool window_pays(const RP& P) { return ceil_div(P.n, kScatterT * kScatterPP) >= 6 * scatter_ctas(); }
+
 template <class FT>
 inpc_status launch_scatter(const RP& P, const float* pos, const float* opacity, const FT* feat, const RasterWs& ws,
                            cudaStream_t s) {
-  constexpr int kT = 512, kPP = 2;
-  const long long chunks = ceil_div(P.n, kT * kPP), resident = (long long)device_sm_count() * 2;
-  if (chunks >= 6 * resident && 4 * P.n >= 12 * P.n_pix) {
-    constexpr size_t smem = sizeof(ScatterSmem<kT, kPP>);
+  const bool window = window_pays(P);
+  if (window) {
+    constexpr size_t smem = sizeof(ScatterSmem<kScatterT, kScatterPP>);
     static SmemOnce once;
-    INPC_TRY(set_smem(k_pix_scatter<kT, kPP, FT>, smem, once));
+    INPC_TRY(set_smem(k_pix_scatter<kScatterT, kScatterPP, FT>, smem, once));
     INPC_TIMED("k_pix_scatter", s,
-               k_pix_scatter<kT, kPP, FT><<<(unsigned)resident, kT, smem, s>>>(P, pos, opacity, feat, ws));
-  } else {
-    INPC_TIMED("k_pix_scatter", s,
-               k_pix_scatter_direct<FT><<<point_grid(P.n), 256, 0, s>>>(P, pos, opacity, feat, ws.pix_start,
-                                                                        ws.pix_count, ws.keys, ws.alpha, ws.porg,
-                                                                        ws.pexp));
+               k_pix_scatter<kScatterT, kScatterPP, FT><<<(unsigned)scatter_ctas(), kScatterT, smem, s>>>(
+                   P, pos, opacity, feat, ws));
+    INPC_TRY(check_launch("k_pix_scatter"));
   }
-  return check_launch("k_pix_scatter");
+  INPC_TIMED("k_pix_scatter", s,
+             k_pix_scatter_direct<FT><<<point_grid(P.n), 256, 0, s>>>(P, pos, opacity, feat, ws.pix_start, ws.pix_count,
+                                                                      ws.keys, ws.alpha, ws.porg, ws.pexp,
+                                                                      window ? ws.sample : nullptr));
+  return check_launch("k_pix_scatter_direct");
 }
 
 // Forward binning: per-pixel counts, offsets, buckets (keys and alphas),
@@ -2187,8 +2199,8 @@ inpc_status bin_fragments(const RP& P, const float* pos, const float* opacity, c
                           ClassCaps cap, cudaStream_t s) {
   INPC_CUDA(cudaMemsetAsync(ws.pix_count, 0, sizeof(uint32_t) * P.n_pix, s), "clear pixel counts");
   if (P.n > 0) {
-    INPC_TRY(P.n >= (long long)device_sm_count() * 2048 ? (launch_count<512, 2>(P, pos, ws, s))
-                                                        : (launch_count<256, 1>(P, pos, ws, s)));
+    INPC_TRY(P.n >= (long long)device_sm_count() * 2048 ? (launch_count<512, 2>(P, pos, ws, window_pays(P) ? ws.sample : nullptr, s))
+                                                        : (launch_count<256, 1>(P, pos, ws, nullptr, s)));
   }
   INPC_TRY((scan::run<uint32_t, CountLoad, false>(CountLoad{ws.pix_count}, P.n_pix, ws.pix_start, ws.tops, s)));
   const long long nb = ceil_div(P.n_pix, scan::kBlock);

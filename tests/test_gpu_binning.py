@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,layout", [(1, "uniform"), (255, "uniform"), (257, "pixel"), (1_023, "border"),
-                                      (5_000, "uniform"), (320_001, "uniform"), (320_001, "grouped")])
+                                      (5_000, "uniform"), (320_001, "uniform"), (320_001, "grouped"),
+                                      (1_900_001, "uniform"), (1_900_001, "grouped")])
 def test_binned_fragments_match_oracle(gpu, oracle, n, layout):
     rng = np.random.default_rng(n)
     W, H, F = 331, 203, 4
