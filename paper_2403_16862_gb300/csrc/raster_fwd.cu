@@ -31,12 +31,11 @@ extern "C" inpc_status inpc_rasterize_fwd(const inpc_camera* cam, const inpc_ras
   const size_t va = P.F % 4 == 0 ? (P.bf16 && P.F != 64 ? 8 : 16) : (P.bf16 ? 2 : 4);
   if (!aligned(feat, va) || !aligned(image, va) || !aligned(pos, 4))
     return fail(INPC_ERR_INVALID_ARG, "feat/image must be %zu-byte aligned", va);
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const RasterFwdCall call{cam, opts, pos, opacity, feat, n, image, T_final, n_contrib, workspace, s};
+  const RasterFwdCall call{cam,   opts,    pos,       opacity,   feat, n,
+                           image, T_final, n_contrib, workspace, reinterpret_cast<cudaStream_t>(stream)};
   return dispatch(P.F, [&](auto, auto Gc) -> inpc_status {
     constexpr int GA = decltype(Gc)::value;
     if (P.bf16 && GA != 32) return fail(INPC_ERR_UNSUPPORTED, "BF16 features need n_channels = 32, 64 or 128");
-    INPC_CUDA(cudaMemsetAsync(workspace, 0, kHeaderBytes, s), "clear header");
     if (P.bf16) return raster_fwd_bf16(call);
     return GA <= 4 ? raster_fwd_narrow4(call) : GA < 32 ? raster_fwd_narrow16(call) : raster_fwd_wide(call);
   });

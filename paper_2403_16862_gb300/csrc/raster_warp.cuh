@@ -285,6 +285,7 @@ template <int V, int GA, class FT>
 __global__ void __launch_bounds__(kThreads, 3) k_blend_fwd_warp(RP P, const FT* __restrict__ feat, RasterWs ws,
                                                                 FT* __restrict__ image, float* __restrict__ T_final,
                                                                 int32_t* __restrict__ n_contrib) {
+  start_next();
   __shared__ WarpCand cand[kWarps];
   const Group<32> G;
   WarpCand& S = cand[threadIdx.x >> 5];
