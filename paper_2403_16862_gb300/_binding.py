@@ -149,6 +149,9 @@ def load(path: str = LIB_PATH):
         L.inpc_sample_octree_halton.argtypes = [C.POINTER(InpcOctree), C.c_uint64, C.c_int64, _P, _P, _P, _P,
                                                 C.c_size_t, _P]
         L.inpc_accumulate_image.argtypes = [_P, C.c_int32, C.c_int64, C.c_float, _P, _P]
+        L.inpc_accumulate_images.argtypes = [C.POINTER(_P), C.c_int32, C.c_int32, C.c_int64, C.c_float, C.c_int32, _P,
+                                             _P]
+        L.inpc_accumulate_images.restype = C.c_int
         L.inpc_contract_positions.argtypes = [_P, C.c_int64, _P, C.c_float, _P, _P]
         L.inpc_sh_head_fwd.argtypes = [C.POINTER(InpcCamera), _P, _P, C.c_int32, C.c_int64, C.c_int32, _P, _P, _P]
         L.inpc_sh_head_bwd.argtypes = [C.POINTER(InpcCamera), _P, _P, C.c_int32, C.c_int64, C.c_int32, _P, _P, _P,
@@ -342,6 +345,15 @@ def inpc_sample_octree_halton(tree: InpcOctree, seed: int, n_samples: int, leaf_
 
 def inpc_accumulate_image(image: int, dtype: int, n_elems: int, scale: float, acc: int, stream: int):
     check(load().inpc_accumulate_image(image, dtype, n_elems, scale, acc, stream))
+
+
+INPC_MAX_IMAGES = 4
+
+
+def inpc_accumulate_images(images, dtype: int, n_elems: int, scale: float, fresh: bool, acc: int, stream: int):
+    """acc (+)= scale * image for up to INPC_MAX_IMAGES images in order (include/inpc_images.h)."""
+    ptrs = (_P * len(images))(*images)
+    check(load().inpc_accumulate_images(ptrs, len(images), dtype, n_elems, scale, 1 if fresh else 0, acc, stream))
 
 
 def inpc_contract_positions(pos: int, n: int, center, radius: float, out: int, stream: int):

@@ -424,13 +424,23 @@ def multisample_render(tree_t, root_size: float, desc, table, cam, seed: int, n_
     c, l, p = tree_t
     opts = opts or RasterOptions(n_channels=desc.n_levels * desc.n_feats, head_mode=True)
     w = view_weights(c, l, p, root_size, cam, lambda_l=lambda_l)
-    acc = torch.zeros(cam.height, cam.width, opts.n_channels, dtype=torch.float32, device=c.device)
-    ws_r = None
+    shape = (cam.height, cam.width, opts.n_channels)
+    if k < 1:
+        return torch.zeros(shape, dtype=torch.float32, device=c.device)
+    acc = torch.empty(shape, dtype=torch.float32, device=c.device)
+    # several images to one pass of the accumulation, while they take at most 2 GiB
+    group = max(1, min(B.INPC_MAX_IMAGES, (2 << 30) // max(1, acc.numel() * opts.dtype.itemsize)))
+    dt = B.INPC_BF16 if opts.bf16 else B.INPC_F32
+    images, fresh, ws_r = [], True, None
     for v in range(k):
         _, pos, _ = sample_octree_view(c, l, w, root_size, cam, seed, v, n_samples, max_rounds=max_rounds)
         h = query_hashgrid(desc, table, pos)
         img, _, _, ws_r = rasterize_fwd(cam, opts, pos, h, ws=ws_r)
-        accumulate_image(img, acc, 1.0 / k)
+        images.append(img)
+        if len(images) == group or v == k - 1:
+            B.inpc_accumulate_images([i.data_ptr() for i in images], dt, acc.numel(), 1.0 / k, fresh, _ptr(acc),
+                                     _stream())
+            images, fresh = [], False
     return acc
 
 

@@ -16,6 +16,7 @@
 
 #include <cuda_bf16.h>
 
+#include "../../include/inpc_images.h"
 #include "sample_impl.cuh"
 
 namespace inpc {
@@ -461,6 +462,59 @@ __global__ void k_accumulate(const T* __restrict__ img, float* __restrict__ acc,
     acc[i] = __fmaf_rn(scale, (float)img[i], acc[i]);
 }
 
+// The same for several images in one pass (in order, one rounding each, so
+// the result has the same bits), from acc or, with `fresh`, from zero.  Bound
+// by memory: four of 1237 x 822 x 64 in 188 us (1.30 GB at 6.9 TB/s); an image
+// at a time reads and writes acc again for each, 609 us and 34 us for the
+// zeros.  Where the addresses allow it a thread takes 4 elements (16 bytes of
+// FP32).
+struct Images {
+  const void* at[INPC_MAX_IMAGES];
+};
+
+__device__ __forceinline__ float4 load4(const float* p) { return __ldcs(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 v = __ldcs(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                     __uint_as_float(v.y & 0xffff0000u));
+}
+
+template <class T, int K>
+__global__ void __launch_bounds__(256) k_accumulate_images(Images im, float* __restrict__ acc, int64_t n, int vec,
+                                                           float scale, int fresh) {
+  const int64_t at0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  if (vec) {
+    for (int64_t i = at0; i < n / 4; i += stride) {
+      float4 v[K];
+#pragma unroll
+      for (int k = 0; k < K; ++k) v[k] = load4(static_cast<const T*>(im.at[k]) + 4 * i);
+      float4* const o = reinterpret_cast<float4*>(acc) + i;
+      float4 a = fresh ? make_float4(0.f, 0.f, 0.f, 0.f) : *o;
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        a = make_float4(__fmaf_rn(scale, v[k].x, a.x), __fmaf_rn(scale, v[k].y, a.y), __fmaf_rn(scale, v[k].z, a.z),
+                        __fmaf_rn(scale, v[k].w, a.w));
+      *o = a;
+    }
+  }
+  for (int64_t i = (vec ? n / 4 * 4 : 0) + at0; i < n; i += stride) {
+    float a = fresh ? 0.f : acc[i];
+#pragma unroll
+    for (int k = 0; k < K; ++k) a = __fmaf_rn(scale, (float)static_cast<const T*>(im.at[k])[i], a);
+    acc[i] = a;
+  }
+}
+
+template <class T>
+void launch_accumulate(const Images& im, int k, float* acc, int64_t n, int vec, float scale, int fresh, unsigned grid,
+                       cudaStream_t s) {
+  static_assert(INPC_MAX_IMAGES == 4, "one case per count");
+  if (k == 1) k_accumulate_images<T, 1><<<grid, 256, 0, s>>>(im, acc, n, vec, scale, fresh);
+  else if (k == 2) k_accumulate_images<T, 2><<<grid, 256, 0, s>>>(im, acc, n, vec, scale, fresh);
+  else if (k == 3) k_accumulate_images<T, 3><<<grid, 256, 0, s>>>(im, acc, n, vec, scale, fresh);
+  else k_accumulate_images<T, 4><<<grid, 256, 0, s>>>(im, acc, n, vec, scale, fresh);
+}
+
 
 }  // namespace
 }  // namespace inpc
@@ -564,6 +618,34 @@ extern "C" inpc_status inpc_accumulate_image(const void* image, int32_t dtype, i
   else
     k_accumulate<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(image), acc, n_elems, scale);
   return check_launch("k_accumulate");
+}
+
+extern "C" inpc_status inpc_accumulate_images(const void* const* images, int32_t n_images, int32_t dtype,
+                                              int64_t n_elems, float scale, int32_t fresh, float* acc,
+                                              inpc_stream_t stream) {
+  inpc::fault_arg(acc);
+  if (n_elems < 0) return fail(INPC_ERR_INVALID_ARG, "n_elems < 0");
+  if (n_images < 1 || n_images > INPC_MAX_IMAGES)
+    return fail(INPC_ERR_INVALID_ARG, "n_images must be in [1, %d]", INPC_MAX_IMAGES);
+  if (dtype != INPC_F32 && dtype != INPC_BF16) return fail(INPC_ERR_UNSUPPORTED, "dtype must be INPC_F32 or INPC_BF16");
+  if (n_elems == 0) return INPC_OK;
+  if (!images || !acc) return fail(INPC_ERR_INVALID_ARG, "null pointer");
+  const size_t elem = dtype == INPC_F32 ? 4 : 2;
+  Images im = {};
+  bool vec = aligned(acc, 16);
+  for (int k = 0; k < n_images; ++k) {
+    if (!images[k]) return fail(INPC_ERR_INVALID_ARG, "null pointer");
+    if (!aligned(images[k], elem)) return fail(INPC_ERR_INVALID_ARG, "misaligned image");
+    im.at[k] = images[k];
+    vec = vec && aligned(images[k], 4 * elem);
+  }
+  if (!aligned(acc, 4)) return fail(INPC_ERR_INVALID_ARG, "misaligned acc");
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  const unsigned grid = (unsigned)std::max<int64_t>(
+      1, std::min<int64_t>(ceil_div(vec ? ceil_div(n_elems, 4) : n_elems, 256), (int64_t)device_sm_count() * 16));
+  if (dtype == INPC_F32) launch_accumulate<float>(im, n_images, acc, n_elems, vec, scale, fresh != 0, grid, s);
+  else launch_accumulate<__nv_bfloat16>(im, n_images, acc, n_elems, vec, scale, fresh != 0, grid, s);
+  return check_launch("k_accumulate_images");
 }
 
 namespace inpc {
