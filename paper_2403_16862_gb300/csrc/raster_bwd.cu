@@ -1,5 +1,6 @@
 // raster_bwd.cu -- C ABI of the rasterizer backward (App. A.6).
 #include "adjoint_impl.cuh"
+#include "raster_fwd.h"
 #include "raster_impl.cuh"
 
 namespace inpc {
@@ -252,14 +253,15 @@ extern "C" inpc_status inpc_rasterize_bwd(const inpc_camera* cam, const inpc_ras
   });
 }
 
-extern "C" inpc_status inpc_rasterize_bwd_hashgrid(const inpc_camera* cam, const inpc_raster_opts* opts,
-                                                   const inpc_hashgrid_desc* grid, const float* pos, const void* feat,
-                                                   int64_t n, const float* T_final, const int32_t* n_contrib,
-                                                   const float* d_image, float* grad_table, float* d_feat,
-                                                   void* workspace, size_t workspace_bytes, inpc_stream_t stream) {
+inpc_status inpc::rasterize_bwd_hashgrid(const inpc_camera* cam, const inpc_raster_opts* opts,
+                                         const inpc_hashgrid_desc* grid, const float* pos, const void* feat, int64_t n,
+                                         const float* T_final, const int32_t* n_contrib, const float* d_image,
+                                         float* grad_table, float* d_feat, void* workspace, size_t workspace_bytes,
+                                         inpc_stream_t stream, bool together) {
   inpc::fault_arg(pos);
   RP P;
   INPC_TRY(make_rp(cam, opts, n, P));
+  P.together = together;
   GridParams Gp;
   int64_t n_entries = 0;
   INPC_TRY(make_params(grid, Gp, &n_entries));
@@ -304,6 +306,15 @@ extern "C" inpc_status inpc_rasterize_bwd_hashgrid(const inpc_camera* cam, const
       return run(float());
     }
   });
+}
+
+extern "C" inpc_status inpc_rasterize_bwd_hashgrid(const inpc_camera* cam, const inpc_raster_opts* opts,
+                                                   const inpc_hashgrid_desc* grid, const float* pos, const void* feat,
+                                                   int64_t n, const float* T_final, const int32_t* n_contrib,
+                                                   const float* d_image, float* grad_table, float* d_feat,
+                                                   void* workspace, size_t workspace_bytes, inpc_stream_t stream) {
+  return inpc::rasterize_bwd_hashgrid(cam, opts, grid, pos, feat, n, T_final, n_contrib, d_image, grad_table, d_feat,
+                                      workspace, workspace_bytes, stream, true);
 }
 
 extern "C" inpc_status inpc_rasterize_bwd_hashgrid_workspace_size(const inpc_camera* cam, const inpc_raster_opts* opts,

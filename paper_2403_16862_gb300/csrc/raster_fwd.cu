@@ -15,10 +15,10 @@ extern "C" inpc_status inpc_rasterize_workspace_size(const inpc_camera* cam, con
   return INPC_OK;
 }
 
-extern "C" inpc_status inpc_rasterize_fwd(const inpc_camera* cam, const inpc_raster_opts* opts, const float* pos,
-                                          const float* opacity, const void* feat, int64_t n, void* image,
-                                          float* T_final, int32_t* n_contrib, void* workspace,
-                                          size_t workspace_bytes, inpc_stream_t stream) {
+inpc_status inpc::rasterize_fwd(const inpc_camera* cam, const inpc_raster_opts* opts, const float* pos,
+                                const float* opacity, const void* feat, int64_t n, void* image, float* T_final,
+                                int32_t* n_contrib, void* workspace, size_t workspace_bytes, inpc_stream_t stream,
+                                bool together) {
   inpc::fault_arg(pos);
   RP P;
   INPC_TRY(make_rp(cam, opts, n, P, kMaxFwdPoints));
@@ -32,11 +32,19 @@ extern "C" inpc_status inpc_rasterize_fwd(const inpc_camera* cam, const inpc_ras
   if (!aligned(feat, va) || !aligned(image, va) || !aligned(pos, 4))
     return fail(INPC_ERR_INVALID_ARG, "feat/image must be %zu-byte aligned", va);
   const RasterFwdCall call{cam,   opts,    pos,       opacity,   feat, n,
-                           image, T_final, n_contrib, workspace, reinterpret_cast<cudaStream_t>(stream)};
+                           image, T_final, n_contrib, workspace, reinterpret_cast<cudaStream_t>(stream), together};
   return dispatch(P.F, [&](auto, auto Gc) -> inpc_status {
     constexpr int GA = decltype(Gc)::value;
     if (P.bf16 && GA != 32) return fail(INPC_ERR_UNSUPPORTED, "BF16 features need n_channels = 32, 64 or 128");
     if (P.bf16) return raster_fwd_bf16(call);
     return GA <= 4 ? raster_fwd_narrow4(call) : GA < 32 ? raster_fwd_narrow16(call) : raster_fwd_wide(call);
   });
+}
+
+extern "C" inpc_status inpc_rasterize_fwd(const inpc_camera* cam, const inpc_raster_opts* opts, const float* pos,
+                                          const float* opacity, const void* feat, int64_t n, void* image,
+                                          float* T_final, int32_t* n_contrib, void* workspace,
+                                          size_t workspace_bytes, inpc_stream_t stream) {
+  return inpc::rasterize_fwd(cam, opts, pos, opacity, feat, n, image, T_final, n_contrib, workspace, workspace_bytes,
+                             stream, true);
 }

@@ -7,6 +7,7 @@ namespace inpc {
 inpc_status raster_fwd_wide(const RasterFwdCall& c) {
   RP P;
   INPC_TRY(make_rp(c.cam, c.opts, c.n, P, kMaxFwdPoints));
+  P.together = c.together;
   const RasterWs ws = carve(c.workspace, P.n_pix, c.n);
   return dispatch(P.F, [&](auto Vc, auto Gc) -> inpc_status {
     constexpr int V = decltype(Vc)::value, GA = decltype(Gc)::value;

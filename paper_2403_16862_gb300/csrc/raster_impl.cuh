@@ -75,6 +75,7 @@ struct RP {
   long long n_pix;
   int idb;                  // point-index bits of the sort key
   uint32_t dbase;           // subtracted from the FP32 depth bits in the key
+  int together;             // (host) a pass's blending kernels may overlap (launch_group)
   unsigned long long idm;   // (1 << idb) - 1
 };
 
@@ -2127,6 +2128,7 @@ inpc_status make_rp(const inpc_camera* cam, const inpc_raster_opts* o, int64_t n
   P.alpha_max = o->alpha_max;
   P.n = n;
   P.n_pix = (long long)cam->width * cam->height;
+  P.together = 1;
   return INPC_OK;
 }
 
@@ -2231,13 +2233,13 @@ inpc_status launch_scatter(const RP& P, const float* pos, const float* opacity, 
 }
 
 // Launches a kernel of a group that may run together.  The group's first
-// kernel (with_previous false) starts when the work before it is done; each
+// kernel (with_previous 0) starts when the work before it is done; each
 // later one as soon as the CTAs of the one before have all started (they call
 // start_next first thing).  No kernel of a group reads what another one
 // writes, and each completes after the one before it (finish_previous), so
 // work behind the group waits for all of it.
 template <class... Ps, class... As>
-inpc_status launch_group(void (*kernel)(Ps...), bool with_previous, unsigned grid, size_t smem, cudaStream_t s,
+inpc_status launch_group(void (*kernel)(Ps...), int with_previous, unsigned grid, size_t smem, cudaStream_t s,
                          As... args) {
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -2290,26 +2292,32 @@ inpc_status launch_fwd(const RP& P, const float* pos, const float* opacity, cons
   INPC_TRY(bin_fragments(P, pos, opacity, feat, ws, ClassCaps{2 * GA, 4 * GA, GA * kRegMax}, s));
   static SmemOnce f2;
   INPC_TRY(set_smem(k_blend_fwd_heavy<V, GA, FT>, HeavyBuf::bytes(), f2));
-  // Together, the lists first: a list is a few long chains per SM, and the
-  // tiles fill the rest of the chip beside it.  The CTA path waits for all (it
-  // takes over what the warps leave open).
   const unsigned sm = (unsigned)device_sm_count();
-  INPC_TIMED("k_blend_fwd_warp", s,
-             INPC_TRY(launch_group(k_blend_fwd_warp<V, GA, FT>, false, sm * 3, 0, s, P, feat, ws, image, T_final,
-                                   n_contrib)));
-  INPC_TRY(check_launch("k_blend_fwd_warp"));
-  INPC_TIMED("k_blend_fwd_large", s,
-             INPC_TRY(launch_group(k_blend_fwd_large<V, GA, FT, kRegMax>, true, sm * 3, 0, s, P, feat, ws, image,
-                                   T_final, n_contrib)));
-  INPC_TRY(check_launch("k_blend_fwd_large"));
-  INPC_TIMED("k_blend_fwd_large", s,
-             INPC_TRY(launch_group(k_blend_fwd_large<V, GA, FT, 4>, true, sm * 4, 0, s, P, feat, ws, image, T_final,
-                                   n_contrib)));
-  INPC_TRY(check_launch("k_blend_fwd_large"));
-  INPC_TIMED("k_blend_fwd", s,
-             INPC_TRY(launch_group(k_blend_fwd<V, GA, FT>, true, (unsigned)P.n_tiles, 0, s, P, feat, ws, image,
-                                   T_final, n_contrib)));
-  INPC_TRY(check_launch("k_blend_fwd"));
+  const auto launch = [&](const char* name, auto kernel, unsigned grid, int with_previous) -> inpc_status {
+    INPC_TIMED(name, s,
+               INPC_TRY(launch_group(kernel, with_previous, grid, 0, s, P, feat, ws, image, T_final, n_contrib)));
+    return check_launch(name);
+  };
+  const auto tiles = [&](int w) { return launch("k_blend_fwd", k_blend_fwd<V, GA, FT>, (unsigned)P.n_tiles, w); };
+  const auto mid = [&](int w) { return launch("k_blend_fwd_large", k_blend_fwd_large<V, GA, FT, 4>, sm * 4, w); };
+  const auto wide = [&](int w) { return launch("k_blend_fwd_large", k_blend_fwd_large<V, GA, FT, kRegMax>, sm * 3, w); };
+  const auto warps = [&](int w) { return launch("k_blend_fwd_warp", k_blend_fwd_warp<V, GA, FT>, sm * 3, w); };
+  // Together, the lists first: a list is a few long chains per SM, and the
+  // tiles fill the rest of the chip beside it.  One by one, the tiles first
+  // (32 views of 1M samples over 8 streams 37.9-39.6 ms, the lists first
+  // 40.0-40.4).
+  // The CTA path waits for all (it takes over what the warps leave open).
+  if (P.together) {
+    INPC_TRY(warps(0));
+    INPC_TRY(wide(1));
+    INPC_TRY(mid(1));
+    INPC_TRY(tiles(1));
+  } else {
+    INPC_TRY(tiles(0));
+    INPC_TRY(mid(0));
+    INPC_TRY(wide(0));
+    INPC_TRY(warps(0));
+  }
   INPC_TIMED("k_blend_fwd_heavy", s,
              k_blend_fwd_heavy<V, GA, FT><<<device_sm_count() * 4, kThreads, HeavyBuf::bytes(), s>>>(
                  P, feat, ws, image, T_final, n_contrib));
@@ -2329,20 +2337,25 @@ inpc_status launch_blend_bwd(const RP& P, const FT* feat, const int32_t* n_contr
                  n_contrib, ws.pix_start, P.n_pix, 2 * GA, kCandMax, ws.heavy, ws.heavy_count, ws.large,
                  ws.large_count));
   INPC_TRY(check_launch("k_classify_bwd"));
-  // together, as in the forward
+  // together or one by one, as in the forward
   const unsigned sm = (unsigned)device_sm_count();
-  INPC_TIMED("k_blend_bwd_heavy", s,
-             INPC_TRY(launch_group(k_blend_bwd_heavy<V, GA, FT>, false, sm * 4, HeavyBwdBuf::bytes(), s, P, feat,
-                                   n_contrib, d_image, ws)));
-  INPC_TRY(check_launch("k_blend_bwd_heavy"));
-  INPC_TIMED("k_blend_bwd_large", s,
-             INPC_TRY(launch_group(k_blend_bwd_large<V, GA, FT>, true, sm * 3, 0, s, P, feat, n_contrib, d_image,
-                                   ws)));
-  INPC_TRY(check_launch("k_blend_bwd_large"));
-  INPC_TIMED("k_blend_bwd", s,
-             INPC_TRY(launch_group(k_blend_bwd<V, GA, FT>, true, (unsigned)P.n_tiles, 0, s, P, feat, n_contrib,
-                                   d_image, ws)));
-  return check_launch("k_blend_bwd");
+  const auto launch = [&](const char* name, auto kernel, unsigned grid, size_t smem, int with_previous) -> inpc_status {
+    INPC_TIMED(name, s, INPC_TRY(launch_group(kernel, with_previous, grid, smem, s, P, feat, n_contrib, d_image, ws)));
+    return check_launch(name);
+  };
+  const auto tiles = [&](int w) { return launch("k_blend_bwd", k_blend_bwd<V, GA, FT>, (unsigned)P.n_tiles, 0, w); };
+  const auto lists = [&](int w) { return launch("k_blend_bwd_large", k_blend_bwd_large<V, GA, FT>, sm * 3, 0, w); };
+  const auto heavy = [&]() {
+    return launch("k_blend_bwd_heavy", k_blend_bwd_heavy<V, GA, FT>, sm * 4, HeavyBwdBuf::bytes(), 0);
+  };
+  if (P.together) {
+    INPC_TRY(heavy());
+    INPC_TRY(lists(1));
+    return tiles(1);
+  }
+  INPC_TRY(tiles(0));
+  INPC_TRY(lists(0));
+  return heavy();
 }
 
 template <int V, int GA, class FT>
