@@ -1190,7 +1190,9 @@ __device__ __forceinline__ long long tile_pixel_index(const RP& P, int tx, int t
 }
 
 // The background (zero color, T = 1, no fragment) of the tile's empty
-// pixels, one warp per pixel.
+// pixels, one warp per pixel: 8 bytes per store where F is a multiple of 4
+// (the image is then aligned to 8 bytes or more), else one channel (FP32, of
+// which the entry asks no more than 4-byte alignment).
 template <class FT>
 __device__ __forceinline__ void fill_empty(const RP& P, int tx, int ty, const TileSmem& S, FT* __restrict__ image,
                                            float* __restrict__ T_final, int32_t* __restrict__ n_contrib) {
@@ -1200,7 +1202,7 @@ __device__ __forceinline__ void fill_empty(const RP& P, int tx, int ty, const Ti
     if (S.m[j] != 0) continue;
     const long long q = tile_pixel_index(P, tx, ty, j);
     char* row = reinterpret_cast<char*>(image + q * P.F);
-    if (bytes % 8 == 0) {
+    if (P.F % 4 == 0) {
       for (int u = lane; u < bytes / 8; u += 32) reinterpret_cast<uint2*>(row)[u] = make_uint2(0u, 0u);
     } else {
       for (int u = lane; u < bytes / 4; u += 32) reinterpret_cast<uint32_t*>(row)[u] = 0u;
