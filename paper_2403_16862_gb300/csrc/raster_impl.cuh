@@ -93,9 +93,9 @@ struct RasterWs {
   uint32_t* status;
   uint32_t* heavy_count;     // header word 1
   uint32_t* large_count;     // header word 2
-  uint32_t* large_next;      // header word 3: the list kernel's next list entry (forward, then backward)
+  uint32_t* large_next;      // header word 3: the list kernel's next list entry
   uint32_t* heavy_next;      // header word 4: the forward CTA kernel's next list entry
-  uint32_t* wide_count;      // header word 5: forward list entries with 8 registers per lane (at the list's end)
+  uint32_t* wide_count;      // header word 5: entries at the list's end
   uint32_t* wide_next;       // header word 6: their cursor
   uint32_t* select_count;    // header word 7: pixels with a selection by one warp (the front of mid)
   uint32_t* warp_count;      // header word 8: pixels with a whole bucket for one warp (the back of mid)
@@ -105,7 +105,8 @@ struct RasterWs {
   uint32_t* pix_start;       // [n_pix + 1]
   uint32_t* tops;            // prefix-sum block totals
   uint32_t* heavy;           // [n_pix] pixels on the CTA path
-  uint32_t* large;           // [n_pix] pixels with 4 or 8 registers per lane
+  uint32_t* large;           // [n_pix] forward: pixels with 4 (front) or 8 (end) registers per lane; backward: pixels
+                             // for one warp (front) or one lane group (end) each
   uint32_t* mid;             // [n_pix] pixels blended by one warp each (raster_warp.cuh)
   unsigned long long* keys;  // [4n] bucketed fragment keys
   float* alpha;              // [4n] fragment alphas
@@ -273,17 +274,19 @@ __global__ void __launch_bounds__(kClassThreads) k_classify(long long n_pix, Cla
 }
 
 // Backward classes by blended count (the forward's n_contrib, clamped to the
-// bucket): the tile kernel takes nb <= cap_small, the list kernels the rest.
-__global__ void k_classify_bwd(const int32_t* __restrict__ n_contrib, const uint32_t* __restrict__ pix_start,
-                               long long n_pix, uint32_t cap_small, uint32_t cap_large, uint32_t* __restrict__ heavy,
-                               uint32_t* heavy_count, uint32_t* __restrict__ large, uint32_t* large_count) {
+// bucket): the tile kernel takes nb <= cap.small, a lane group per pixel (the
+// back of the list) nb <= cap.large, a warp per pixel (its front) nb <=
+// kCandMax, the CTA path the rest.
+__global__ void k_classify_bwd(const int32_t* __restrict__ n_contrib, long long n_pix, ClassCaps cap, RasterWs ws) {
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (q >= n_pix) return;
   const int c = n_contrib[q];
-  const uint32_t m = pix_start[q + 1] - pix_start[q];
+  const uint32_t m = ws.pix_start[q + 1] - ws.pix_start[q];
   const uint32_t nb = c < 0 ? 0u : min((uint32_t)c, m);
-  if (nb > cap_large) heavy[atomicAdd(heavy_count, 1u)] = (uint32_t)q;
-  else if (nb > cap_small) large[atomicAdd(large_count, 1u)] = (uint32_t)q;
+  if (nb <= cap.small) return;
+  if (nb <= cap.large) ws.large[n_pix - 1 - atomicAdd(ws.wide_count, 1u)] = (uint32_t)q;
+  else if (nb <= (uint32_t)kCandMax) ws.large[atomicAdd(ws.large_count, 1u)] = (uint32_t)q;
+  else ws.heavy[atomicAdd(ws.heavy_count, 1u)] = (uint32_t)q;
 }
 
 __device__ __forceinline__ int blended_count(const int32_t* __restrict__ n_contrib, long long q, int m) {
@@ -1402,31 +1405,76 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_bwd(RP P, const FT* __res
 namespace inpc {
 namespace {
 
+// Blended fragments that the backward's lists leave to one lane group of GA
+// lanes; up to kCandMax a warp takes a pixel.  Where most pixels blend a few
+// fragments, a warp each is mostly idle lanes (4 channels, 1.96M points on
+// 1400 x 1400 pixels: backward 1284 us with warps only, 523 us with groups; 8
+// channels 970 and 650; 16 channels, 5.88M points 2278 and 1605).  Groups of 8
+// and 16 lanes gain nothing over warps, and 8 registers a lane pay for single
+// lanes only (16 channels, 4M points on 1000 x 700 pixels: 994 us with 4,
+// 1286 us with 8).
+template <int GA>
+constexpr uint32_t bwd_group_cap() {
+  return GA == 1 || GA == 32 ? GA * kRegMax : GA <= 4 ? 4 * GA : 2 * GA;
+}
+
+// Fewer pixels than this go to warps as well: a group's chain through its
+// fragments is then the time of the launch (4 channels, 64 x 64 pixels: 46 us
+// with groups, 26 us with warps; the lines cross at 20,000 to 50,000 pixels).
+constexpr uint32_t kBwdGroupMin = 32768;
+
+// The list's back, one lane group per pixel.
+template <int V, int GA, class FT>
+__device__ __forceinline__ void bwd_groups(const RP& P, const FT* __restrict__ feat,
+                                           const int32_t* __restrict__ n_contrib, const float* __restrict__ d_image,
+                                           const RasterWs& ws, uint32_t n_group) {
+  const Group<GA> G;
+  for (;;) {
+    uint32_t h = 0;
+    if (G.lg == 0) h = atomicAdd(ws.wide_next, 1u);
+    h = G.bcast(h, 0);
+    if (h >= n_group) break;
+    const long long q = ws.large[P.n_pix - 1 - h];
+    const uint32_t s0 = ws.pix_start[q];
+    const int m = (int)(ws.pix_start[q + 1] - s0);
+    const int nb = blended_count(n_contrib, q, m);
+    if (bwd_group_cap<GA>() == 4 * GA || nb <= 4 * GA)
+      blend_bwd_reg<V, GA, FT, 4>(G, P, ws, s0, m, nb, q, feat, d_image);
+    else
+      blend_bwd_reg<V, GA, FT, kRegMax>(G, P, ws, s0, m, nb, q, feat, d_image);
+  }
+}
+
 template <int V, int GA, class FT>
 __global__ void __launch_bounds__(kThreads, 3) k_blend_bwd_large(RP P, const FT* __restrict__ feat,
                                                                const int32_t* __restrict__ n_contrib,
                                                                const float* __restrict__ d_image, RasterWs ws) {
   start_next();
-  const Group<32> G;  // one warp per pixel
-  const uint32_t n_large = *ws.large_count;
-  // as in the forward list kernel, each group takes the next pixel when done
-  for (;;) {
-    uint32_t h = 0;
-    if (G.lg == 0) h = atomicAdd(ws.large_next, 1u);
-    h = G.bcast(h, 0);
-    if (h >= n_large) break;
-    const long long q = ws.large[h];
-    const uint32_t s0 = ws.pix_start[q];
-    const int m = (int)(ws.pix_start[q + 1] - s0);
-    const int nb = blended_count(n_contrib, q, m);
-    if constexpr (GA < 32) {
-      if (nb <= 64) blend_bwd_warp<V, GA, FT, 2>(G, P, ws, s0, m, nb, q, feat, d_image);
+  // as in the forward list kernel, each group takes the next pixel when done;
+  // the longer chains go first
+  const uint32_t n_group = *ws.wide_count;
+  if constexpr (GA < 32) {
+    const Group<32> G;
+    const uint32_t n_front = *ws.large_count, n_warp = n_front + (n_group < kBwdGroupMin ? n_group : 0u);
+    for (;;) {
+      uint32_t h = 0;
+      if (G.lg == 0) h = atomicAdd(ws.large_next, 1u);
+      h = G.bcast(h, 0);
+      if (h >= n_warp) break;
+      const long long q = ws.large[h < n_front ? h : P.n_pix - 1 - (h - n_front)];
+      const uint32_t s0 = ws.pix_start[q];
+      const int m = (int)(ws.pix_start[q + 1] - s0);
+      const int nb = blended_count(n_contrib, q, m);
+      // one register a lane where a row is one or two lanes (12M points of 8
+      // channels on 1000 x 700 pixels: 1528 -> 1381 us; no gain from 12 on)
+      if (GA <= 2 && nb <= 32) blend_bwd_warp<V, GA, FT, 1>(G, P, ws, s0, m, nb, q, feat, d_image);
+      else if (nb <= 64) blend_bwd_warp<V, GA, FT, 2>(G, P, ws, s0, m, nb, q, feat, d_image);
       else if (nb <= 128) blend_bwd_warp<V, GA, FT, 4>(G, P, ws, s0, m, nb, q, feat, d_image);
       else blend_bwd_warp<V, GA, FT, 8>(G, P, ws, s0, m, nb, q, feat, d_image);
-    } else {
-      if (nb <= 4 * GA) blend_bwd_reg<V, GA, FT, 4>(G, P, ws, s0, m, nb, q, feat, d_image);
-      else blend_bwd_reg<V, GA, FT, kRegMax>(G, P, ws, s0, m, nb, q, feat, d_image);
     }
+  }
+  if constexpr (bwd_group_cap<GA>() > 2 * GA) {
+    if (GA == 32 || n_group >= kBwdGroupMin) bwd_groups<V, GA, FT>(P, feat, n_contrib, d_image, ws, n_group);
   }
   finish_previous();
 }
@@ -2331,13 +2379,12 @@ inpc_status launch_blend_bwd(const RP& P, const FT* feat, const int32_t* n_contr
                              const RasterWs& ws, cudaStream_t s) {
   // fragments that were not blended keep zero scalars
   INPC_CUDA(cudaMemsetAsync(ws.fscal, 0, sizeof(float2) * std::max<long long>(4 * P.n, 1), s), "clear fscal");
-  // the class counts and the list cursors (header words 1-4; the forward's
+  // the class counts and the list cursors (header words 1-6; the forward's
   // kernels are done with them)
-  INPC_CUDA(cudaMemsetAsync(ws.heavy_count, 0, 4 * sizeof(uint32_t), s), "clear class counts");
+  INPC_CUDA(cudaMemsetAsync(ws.heavy_count, 0, 6 * sizeof(uint32_t), s), "clear class counts");
+  const ClassCaps cap{2 * GA, 4 * GA, bwd_group_cap<GA>()};
   INPC_TIMED("k_classify_bwd", s,
-             k_classify_bwd<<<(unsigned)ceil_div(P.n_pix, 256), 256, 0, s>>>(
-                 n_contrib, ws.pix_start, P.n_pix, 2 * GA, kCandMax, ws.heavy, ws.heavy_count, ws.large,
-                 ws.large_count));
+             k_classify_bwd<<<(unsigned)ceil_div(P.n_pix, 256), 256, 0, s>>>(n_contrib, P.n_pix, cap, ws));
   INPC_TRY(check_launch("k_classify_bwd"));
   // together or one by one, as in the forward
   const unsigned sm = (unsigned)device_sm_count();

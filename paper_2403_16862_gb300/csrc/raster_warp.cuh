@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_blend_fwd_warp(RP P, const FT* 
   }
 }
 
-// Backward of 2 GA < nb <= 256 blended fragments (GA < 32): transmittances as
+// Backward of up to 32 R blended fragments (GA < 32): transmittances as
 // in blend_candidates over the blended prefix the forward recorded, then back
 // to front, each lane holding one fragment of the chunk; the dot products
 // c_k . g by groups of GL lanes.
