@@ -5,10 +5,11 @@
 // kWarpKeys it holds the bucket's depths in registers (32 per lane), finds a
 // depth threshold that the nearest 72 to 128 fragments meet by an
 // interpolating search over warp-wide counts, and takes those.  The fragments
-// taken are sorted in registers on 32-bit keys and blended.  What this does
-// not settle (candidates that do not reach t_min, equal depths, a depth span
-// of 2^24 FP32 values) is left to the CTA path.  No barrier is involved, the
-// bucket is read from memory once, and the pixels of a CTA's warps overlap.
+// taken are sorted in registers on 32-bit keys and blended.  Where those do not
+// order them (equal depths, a depth span of 2^24 FP32 values) the warp sorts a
+// whole bucket on its full keys; a selection is left to the CTA path then, and
+// where it does not reach t_min.  No barrier is involved, the bucket is read
+// from memory once, and the pixels of a CTA's warps overlap.
 //
 // The transmittances are those of the CTA path bit for bit: products over
 // chunks of 32 within blocks of 256 fragments, in the same order.
@@ -27,7 +28,7 @@ struct WarpLanes {
 struct WarpCand {  // the fragments a warp works on
   unsigned long long key[kCandMax];
   float alpha[kCandMax];
-  uint32_t pos[kCandMax];  // bucket position
+  uint32_t pos[kCandMax];  // bucket position; of a whole bucket, which needs none, the sort's exchange space
 };
 
 // Blends fragments: each group of GL lanes takes one fragment's row at a
@@ -99,16 +100,50 @@ __device__ __forceinline__ bool sort_candidates(const Group<32>& G, const RP& P,
   return !__any_sync(0xffffffffu, tie);
 }
 
-// Sorts the C <= 32 R candidates and blends the pixel.  False (nothing
-// written) when the sort leaves it open, or when they do not reach t_min and
-// are not the whole bucket.
-template <int V, int GA, class FT, int R>
+// S.pos = the C candidates in the order of their full keys (the network of
+// bitonic_sort_idx, its indices by shifts and masks).
+__device__ __forceinline__ void warp_sort_full(WarpCand& S, int C) {
+  const int lane = threadIdx.x & 31;
+  for (int e = lane; e < C; e += 32) S.pos[e] = (uint32_t)e;
+  __syncwarp();
+  for (int k = 2; (k >> 1) < C; k <<= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      const int flip = 2 * j == k ? k - 1 : j;
+      for (int q = lane; 2 * q < C + k; q += 32) {
+        const int lo = 2 * q - (q & (j - 1)), hi = lo ^ flip;
+        if (hi < C) {
+          const uint32_t a = S.pos[lo], b = S.pos[hi];
+          if (S.key[a] > S.key[b]) {
+            S.pos[lo] = b;
+            S.pos[hi] = a;
+          }
+        }
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// Sorts the C <= 32 R candidates (kWhole: the whole bucket) and blends
+// the pixel.  False (nothing written) when a selection's sort leaves it open
+// or its candidates do not reach t_min.  A selection is not sorted on full
+// keys: its equal depths are rare, and such pixels become the launch's tail
+// (19,200 pixels of 520 fragments, 64 channels: 84 us, 91 us with them).  Whole
+// buckets are, for they may be all ties: 600,000 points in one plane of depth
+// on 200 x 160 pixels, 8 channels, forward 664 us left to the CTA path, 190 us
+// here; at random depths 143 and 125 us.
+template <int V, int GA, class FT, int R, bool kWhole>
 __device__ __forceinline__ bool blend_candidates(const Group<32>& G, const RP& P, const RasterWs& ws, uint32_t s0,
-                                                 int C, int m, long long pix, const WarpCand& S,
+                                                 int C, long long pix, WarpCand& S,
                                                  const FT* __restrict__ feat, FT* __restrict__ image,
                                                  float* __restrict__ T_final, int32_t* __restrict__ n_contrib) {
   uint32_t k[R];
-  if (!sort_candidates<R>(G, P, S, C, k)) return false;
+  if (!sort_candidates<R>(G, P, S, C, k)) {
+    if constexpr (!kWhole) return false;
+    warp_sort_full(S, C);
+#pragma unroll
+    for (int r = 0; r < R; ++r) k[r] = r * 32 + G.lg < C ? S.pos[r * 32 + G.lg] : 0xFFu;
+  }
   uint32_t id[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) id[r] = r * 32 + G.lg < C ? (uint32_t)(S.key[k[r] & 255u] & P.idm) : 0u;
@@ -138,11 +173,11 @@ __device__ __forceinline__ bool blend_candidates(const Group<32>& G, const RP& P
       T = __shfl_sync(0xffffffffu, Tn, take - 1);
     }
   }
-  if (!stop && C != m) return false;
+  if (!kWhole && !stop) return false;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int j = r * 32 + G.lg;
-    if (j < cnt) ws.order[s0 + j] = make_uint2(S.pos[k[r] & 255u], id[r]);
+    if (j < cnt) ws.order[s0 + j] = make_uint2(kWhole ? k[r] & 255u : S.pos[k[r] & 255u], id[r]);
   }
   if constexpr (V == 2) {  // F = 64
     float acc[16];
@@ -187,13 +222,12 @@ __device__ __forceinline__ bool blend_whole(const Group<32>& G, const RP& P, con
   for (int e = G.lg; e < m; e += 32) {
     S.key[e] = ws.keys[s0 + e];
     S.alpha[e] = ws.alpha[s0 + e];
-    S.pos[e] = (uint32_t)e;
   }
   __syncwarp();
-  if (m <= 32) return blend_candidates<V, GA, FT, 1>(G, P, ws, s0, m, m, q, S, feat, image, T_final, n_contrib);
-  if (m <= 64) return blend_candidates<V, GA, FT, 2>(G, P, ws, s0, m, m, q, S, feat, image, T_final, n_contrib);
-  if (m <= 128) return blend_candidates<V, GA, FT, 4>(G, P, ws, s0, m, m, q, S, feat, image, T_final, n_contrib);
-  return blend_candidates<V, GA, FT, 8>(G, P, ws, s0, m, m, q, S, feat, image, T_final, n_contrib);
+  if (m <= 32) return blend_candidates<V, GA, FT, 1, true>(G, P, ws, s0, m, q, S, feat, image, T_final, n_contrib);
+  if (m <= 64) return blend_candidates<V, GA, FT, 2, true>(G, P, ws, s0, m, q, S, feat, image, T_final, n_contrib);
+  if (m <= 128) return blend_candidates<V, GA, FT, 4, true>(G, P, ws, s0, m, q, S, feat, image, T_final, n_contrib);
+  return blend_candidates<V, GA, FT, 8, true>(G, P, ws, s0, m, q, S, feat, image, T_final, n_contrib);
 }
 
 // The fragments with a depth field of at most t, in bucket order, into S.
@@ -271,7 +305,7 @@ __device__ __forceinline__ bool blend_selected(const Group<32>& G, const RP& P, 
   }
   if (C == 0) return false;  // equal depths make the count jump over the window
   take_front(G, ws, s0, d, m, t, C, S);
-  return blend_candidates<V, GA, FT, 4>(G, P, ws, s0, C, m, q, S, feat, image, T_final, n_contrib);
+  return blend_candidates<V, GA, FT, 4, false>(G, P, ws, s0, C, q, S, feat, image, T_final, n_contrib);
 }
 
 // The warps' launch: the pixels with 8 GA < m <= kCandMax fragments (GA < 32;
