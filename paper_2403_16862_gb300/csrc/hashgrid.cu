@@ -81,11 +81,13 @@ __global__ void __launch_bounds__(256) k_hash_fwd(GridParams P, LevelGroups LG, 
 // point and level with eight reductions each before).  A CTA takes `chunk`
 // consecutive points, its point slots interleaved over them; each lane loads
 // its next point's position and gradient row before it works on the current
-// one.
+// one.  n_coarse (at most kH): the coarse warps' levels; fewer than kH only
+// with coarse_only.
 template <int GA>
 __global__ void __launch_bounds__(256, 4) k_hash_bwd(GridParams P, const float* __restrict__ pos,
                                                      const float4* __restrict__ dh, long long n,
-                                                     float* __restrict__ grad, long long chunk, int coarse_only) {
+                                                     float* __restrict__ grad, long long chunk, int n_coarse,
+                                                     int coarse_only) {
   constexpr int kH = GA / 2;           // levels per half
   constexpr int kPW = 16 / kH;         // points per warp
   constexpr int kGroups = 4 * kPW;     // points in flight per CTA (4 warp pairs)
@@ -97,7 +99,7 @@ __global__ void __launch_bounds__(256, 4) k_hash_bwd(GridParams P, const float* 
   const int lvl = (lane >> 1) % kH;
   const int l = (coarse ? 0 : kH) + lvl;
   const int slot = (warp >> 1) * kPW + lane / (2 * kH);
-  if (l >= P.n_levels || (!coarse && coarse_only)) return;  // nothing below is collective
+  if (coarse ? l >= n_coarse : l >= P.n_levels || coarse_only) return;  // nothing below is collective
   const uint64_t keep = l2_evict_last(), stream = l2_evict_first();
   AdjointLane<kStride> adj(P, l, true, grad, bx, &acc_s[0][(slot * kH + lvl) * 2 + bx]);
   const long long last = min((long long)(blockIdx.x + 1) * chunk, n);
@@ -126,21 +128,55 @@ __global__ void __launch_bounds__(256, 4) k_hash_bwd(GridParams P, const float* 
   if (coarse) adj.flush(keep);
 }
 
+// How the adjoint takes the levels: the first n_coarse on the coarse warps; the
+// others on the fine warps or, with split, level group by level group in a
+// launch of their own.  What is reduced into at a time has to stay in L2 (129
+// MB): the coarse levels within 96 MB, the fine ones within kQueryL2Budget, all
+// of them within 112 MB, counting the rows that the points can touch (8 a level
+// each; a 16-byte row takes a 32-byte sector while its neighbour is not).
+// Random positions, before and after this rule (levels, log2 of the rows):
+// 1,000,000 points 9/21 690 and 370 us, 12/20 677 and 431, 24/19 1482 and 776,
+// 16/19 and 16/21 the same; 1,000 points 16/20 11.0 and 6.1, 32/19 13.2 and 6.3.
+struct AdjointPlan {
+  int n_coarse;
+  bool split;
+};
+
+AdjointPlan plan_adjoint(const GridParams& P, int kH, long long n) {
+  constexpr long long kCoarseBytes = 96ll << 20, kAllBytes = 112ll << 20;
+  const auto bytes = [&](int l, int per_row) {
+    return std::min<long long>(16 * level_rows(P, l), 8 * per_row * n);
+  };
+  AdjointPlan a = {0, false};
+  for (long long coarse = 0; a.n_coarse < kH; ++a.n_coarse) {
+    coarse += bytes(a.n_coarse, 32);
+    if (a.n_coarse > 0 && coarse > kCoarseBytes) break;
+  }
+  long long fine = 0, all = 0;
+  for (int l = 0; l < P.n_levels; ++l) {
+    if (l >= a.n_coarse) fine += bytes(l, 32);
+    all += bytes(l, 16);
+  }
+  a.split = a.n_coarse < kH || fine > kQueryL2Budget || all > kAllBytes;
+  return a;
+}
+
 template <int GA>
 inpc_status launch_hash_bwd(const GridParams& P, const float* pos, const float4* dh, long long n, float* grad,
                             cudaStream_t s) {
   constexpr int kH = GA / 2, kGroups = 4 * (16 / kH);
-  // fine levels beyond the L2 budget go level group by level group
-  const bool split = P.n_levels > kH && !grad_levels_fit_l2(P, kH);
+  const AdjointPlan plan = plan_adjoint(P, kH, n);
   // whole waves of resident CTAs (4 per SM), about 48 points per slot: long
   // enough runs to merge, and no nearly empty last wave
   const long long resident = (long long)device_sm_count() * 4;
   const long long waves = std::max<long long>(1, (n + 24 * kGroups * resident) / (48 * kGroups * resident));
   const long long chunk = kGroups * std::max<long long>(1, ceil_div(n, kGroups * resident * waves));
   INPC_TIMED("k_hash_bwd", s,
-             k_hash_bwd<GA><<<(unsigned)ceil_div(n, chunk), 256, 0, s>>>(P, pos, dh, n, grad, chunk, split ? 1 : 0));
+             k_hash_bwd<GA><<<(unsigned)ceil_div(n, chunk), 256, 0, s>>>(P, pos, dh, n, grad, chunk, plan.n_coarse,
+                                                                     plan.split ? 1 : 0));
   INPC_TRY(check_launch("k_hash_bwd"));
-  return split ? launch_grad_levels(P, kH, pos, dh + kH, P.n_levels, 1, n, grad, s) : INPC_OK;
+  if (!plan.split) return INPC_OK;
+  return launch_grad_levels(P, plan.n_coarse, pos, dh + plan.n_coarse, P.n_levels, 1, n, grad, s);
 }
 
 }  // namespace
