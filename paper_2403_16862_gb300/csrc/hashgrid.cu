@@ -81,13 +81,13 @@ __global__ void __launch_bounds__(256) k_hash_fwd(GridParams P, LevelGroups LG, 
 // point and level with eight reductions each before).  A CTA takes `chunk`
 // consecutive points, its point slots interleaved over them; each lane loads
 // its next point's position and gradient row before it works on the current
-// one.  n_coarse (at most kH): the coarse warps' levels; fewer than kH only
-// with coarse_only.
+// one.  The coarse warps take levels 0 .. n_coarse - 1 (at most kH), the fine
+// warps levels kH .. l_end - 1 (none with l_end = 0).
 template <int GA>
 __global__ void __launch_bounds__(256, 4) k_hash_bwd(GridParams P, const float* __restrict__ pos,
                                                      const float4* __restrict__ dh, long long n,
                                                      float* __restrict__ grad, long long chunk, int n_coarse,
-                                                     int coarse_only) {
+                                                     int l_end) {
   constexpr int kH = GA / 2;           // levels per half
   constexpr int kPW = 16 / kH;         // points per warp
   constexpr int kGroups = 4 * kPW;     // points in flight per CTA (4 warp pairs)
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256, 4) k_hash_bwd(GridParams P, const float* 
   const int lvl = (lane >> 1) % kH;
   const int l = (coarse ? 0 : kH) + lvl;
   const int slot = (warp >> 1) * kPW + lane / (2 * kH);
-  if (coarse ? l >= n_coarse : l >= P.n_levels || coarse_only) return;  // nothing below is collective
+  if (l >= (coarse ? n_coarse : l_end)) return;  // nothing below is collective
   const uint64_t keep = l2_evict_last(), stream = l2_evict_first();
   AdjointLane<kStride> adj(P, l, true, grad, bx, &acc_s[0][(slot * kH + lvl) * 2 + bx]);
   const long long last = min((long long)(blockIdx.x + 1) * chunk, n);
@@ -173,7 +173,7 @@ inpc_status launch_hash_bwd(const GridParams& P, const float* pos, const float4*
   const long long chunk = kGroups * std::max<long long>(1, ceil_div(n, kGroups * resident * waves));
   INPC_TIMED("k_hash_bwd", s,
              k_hash_bwd<GA><<<(unsigned)ceil_div(n, chunk), 256, 0, s>>>(P, pos, dh, n, grad, chunk, plan.n_coarse,
-                                                                     plan.split ? 1 : 0));
+                                                                     plan.split ? 0 : P.n_levels));
   INPC_TRY(check_launch("k_hash_bwd"));
   if (!plan.split) return INPC_OK;
   return launch_grad_levels(P, plan.n_coarse, pos, dh + plan.n_coarse, P.n_levels, 1, n, grad, s);

@@ -279,14 +279,24 @@ __global__ void __launch_bounds__(kClassThreads) k_classify(long long n_pix, Cla
 // kCandMax, the CTA path the rest.
 __global__ void k_classify_bwd(const int32_t* __restrict__ n_contrib, long long n_pix, ClassCaps cap, RasterWs ws) {
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (q >= n_pix) return;
-  const int c = n_contrib[q];
-  const uint32_t m = ws.pix_start[q + 1] - ws.pix_start[q];
-  const uint32_t nb = c < 0 ? 0u : min((uint32_t)c, m);
-  if (nb <= cap.small) return;
-  if (nb <= cap.large) ws.large[n_pix - 1 - atomicAdd(ws.wide_count, 1u)] = (uint32_t)q;
-  else if (nb <= (uint32_t)kCandMax) ws.large[atomicAdd(ws.large_count, 1u)] = (uint32_t)q;
-  else ws.heavy[atomicAdd(ws.heavy_count, 1u)] = (uint32_t)q;
+  uint32_t nb = 0;
+  if (q < n_pix) {
+    const int c = n_contrib[q];
+    nb = c < 0 ? 0u : min((uint32_t)c, ws.pix_start[q + 1] - ws.pix_start[q]);
+  }
+  // one lane per class goes to its counter, the classes' round trips together
+  const int cls = nb <= cap.small ? 0 : nb <= cap.large ? 1 : nb <= (uint32_t)kCandMax ? 2 : 3;
+  const unsigned in1 = __ballot_sync(0xffffffffu, cls == 1), in2 = __ballot_sync(0xffffffffu, cls == 2),
+                 in3 = __ballot_sync(0xffffffffu, cls == 3), same = cls == 1 ? in1 : cls == 2 ? in2 : in3;
+  if (cls == 0) return;
+  const int lane = threadIdx.x & 31, lead = __ffs(same) - 1;
+  uint32_t at = 0;
+  if (lane == lead)
+    at = atomicAdd(cls == 1 ? ws.wide_count : cls == 2 ? ws.large_count : ws.heavy_count, (uint32_t)__popc(same));
+  at = __shfl_sync(in1 | in2 | in3, at, lead) + __popc(same & ((1u << lane) - 1u));
+  if (cls == 1) ws.large[n_pix - 1 - at] = (uint32_t)q;
+  else if (cls == 2) ws.large[at] = (uint32_t)q;
+  else if (cls == 3) ws.heavy[at] = (uint32_t)q;
 }
 
 __device__ __forceinline__ int blended_count(const int32_t* __restrict__ n_contrib, long long q, int m) {
