@@ -351,12 +351,12 @@ __device__ __forceinline__ bool in_view(const Cam& c, const float* p) {
 // list after each round so that a round's work is dense.  (One launch per
 // round over all slots took 8 x 5.4 us and the final count 6 us for 1M
 // slots, beside the 32 us of k_place.)
-constexpr int kViewTile = 2048;
+constexpr int kViewTile = 2048;  // slots at most (the launch's tile is a multiple of the CTA's threads)
 
 __global__ void __launch_bounds__(256) k_place_view(const uint32_t* __restrict__ starts,
                                                     const uint64_t* __restrict__ cdf,
                                                     const uint32_t* __restrict__ guide, int64_t L, int stride_log2,
-                                                    int Gl, Cam cam, int64_t n, int max_rounds, uint32_t k0,
+                                                    int Gl, Cam cam, int64_t n, int tile, int max_rounds, uint32_t k0,
                                                     uint32_t k1, uint32_t view_id, const float* __restrict__ centers,
                                                     const int32_t* __restrict__ levels, float root_size,
                                                     int32_t* __restrict__ leaf_out, float* __restrict__ pos_out,
@@ -368,8 +368,8 @@ __global__ void __launch_bounds__(256) k_place_view(const uint32_t* __restrict__
   if (threadIdx.x < 2) n_out[threadIdx.x] = 0;
   load_coarse(LdPlain(), starts, L, stride_log2, coarse, n_coarse);
   const uint64_t Qi = cdf[L - 1];
-  for (int64_t t0 = (int64_t)blockIdx.x * kViewTile; t0 < n; t0 += (int64_t)gridDim.x * kViewTile) {
-    const int m0 = (int)min((int64_t)kViewTile, n - t0);
+  for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < n; t0 += (int64_t)gridDim.x * tile) {
+    const int m0 = (int)min((int64_t)tile, n - t0);
     int m = m0, cur = 0;
     for (int r = -1;; ++r, cur ^= 1) {  // r = -1: the slots' first draw
       for (int e = threadIdx.x; e < m; e += blockDim.x) {
@@ -700,10 +700,15 @@ inpc_status sample_impl(const inpc_octree* tree, uint64_t seed, uint32_t view_id
                                                                tree->levels, tree->root_size, leaf_idx_out, pos_out));
       INPC_TRY(check_launch("k_place_halton"));
     } else if (view) {
-      const int64_t tiles = std::min<int64_t>(ceil_div(n_samples, kViewTile), (int64_t)sms * 8);
+      // Four tiles per SM where n allows it: a slot out of view is a chain of
+      // max_rounds draws, so a few large tiles leave the chip idle (most slots
+      // out of view, 4,096 leaves: 8,000 slots 178 us with tiles of 2048 and 91
+      // us with 256, 300,000 slots 183 and 122 us; from 1.2M on the same).
+      const int tile = (int)std::min<int64_t>(kViewTile, 256 * ceil_div(n_samples, (int64_t)sms * 4 * 256));
+      const int64_t tiles = std::min<int64_t>(ceil_div(n_samples, tile), (int64_t)sms * 8);
       INPC_TIMED("k_place_view", s,
                  k_place_view<<<(unsigned)tiles, 256, 0, s>>>(ws.starts, ws.cdf, ws.guide, L, sl, Gl, to_cam(*view),
-                                                              n_samples, max_rounds, k0, k1, view_id, tree->centers,
+                                                              n_samples, tile, max_rounds, k0, k1, view_id, tree->centers,
                                                               tree->levels, tree->root_size, leaf_idx_out, pos_out,
                                                               n_left));
       INPC_TRY(check_launch("k_place_view"));
