@@ -8,6 +8,7 @@
 // blends 4 channels with given opacities) instead of once per splat inside
 // the blend: the point's 37 features are read once, not four times.
 #include <cmath>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -93,15 +94,29 @@ constexpr int kHeadThreads = 128;
 constexpr int kHeadFeats = 37;   // opacity and 36 SH features
 constexpr int kHeadStride = 41;  // shared-memory row of a point (odd: the lanes' rows start in different banks)
 
-// A warp takes 32 consecutive points: it reads their rows' first 37 (kVec:
-// 40, 4 at a time) features side by side into shared memory, then each lane
-// works on its own point.  (One thread per point reading its row directly
-// touched 32 lines per load: 500k points, 64 features, 78 us.)
-template <class HT, bool kVec>
+// How the forward reads the rows (2,000,000 FP32 points, us: a thread per point
+// reading its row with twice as many threads a CTA, as before the warps; through
+// shared memory 4 elements at a time; one at a time; kDirect):
+//   64 features           280, 119, 182, -
+//   64, at an odd offset  280, -, 182, 252
+//   37                    179, -, 277 (175 unrolled), 97
+//   71                    183, -, 292 (186), 131
+enum class Rows {
+  kVec,     // F % 4 == 0, F >= 40 and 4 elements aligned: the first 40 features, 4 at a time
+  kOne,     // F % 4 == 0 otherwise: the first 37, one at a time
+  kDirect,  // F % 4 != 0: each lane its own row (32 lanes' rows lie in different sectors and cache sets)
+};
+
+// A warp takes 32 consecutive points: it reads their rows' first features
+// side by side into shared memory, then each lane works on its own point.  (One
+// thread per point reading its row directly touched 32 lines per load: 500k
+// points, 64 features, 78 us.)
+template <class HT, Rows kRows>
 __global__ void __launch_bounds__(kHeadThreads) k_sh_head_fwd(ShConsts k, const float* __restrict__ pos,
                                                               const HT* __restrict__ h, int64_t n, int F,
                                                               float* __restrict__ alpha, float* __restrict__ color) {
-  __shared__ float rows_s[kHeadThreads / 32][32 * kHeadStride];
+  constexpr bool kDirect = kRows == Rows::kDirect;
+  __shared__ float rows_s[kHeadThreads / 32][kDirect ? 1 : 32 * kHeadStride];
   const int lane = threadIdx.x & 31;
   float* rows = rows_s[threadIdx.x >> 5];
   const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -109,7 +124,7 @@ __global__ void __launch_bounds__(kHeadThreads) k_sh_head_fwd(ShConsts k, const 
     const int64_t p0 = 32 * b;
     const int np = (int)min((int64_t)32, n - p0);
     __syncwarp();
-    if (kVec) {
+    if constexpr (kRows == Rows::kVec) {
 #pragma unroll
       for (int i = 0; i < 10; ++i) {
         const int pt = (i * 32 + lane) / 10, e = 4 * ((i * 32 + lane) % 10);
@@ -122,7 +137,8 @@ __global__ void __launch_bounds__(kHeadThreads) k_sh_head_fwd(ShConsts k, const 
           o[3] = v.w;
         }
       }
-    } else {
+    } else if constexpr (kRows == Rows::kOne) {
+#pragma unroll 8
       for (int i = lane; i < np * kHeadFeats; i += 32)
         rows[i / kHeadFeats * kHeadStride + i % kHeadFeats] = ldf(h + (p0 + i / kHeadFeats) * F + i % kHeadFeats);
     }
@@ -131,14 +147,14 @@ __global__ void __launch_bounds__(kHeadThreads) k_sh_head_fwd(ShConsts k, const 
     const int64_t p = p0 + lane;
     float Y[9];
     sh9(k, pos + 3 * p, Y);
-    const float* row = rows + lane * kHeadStride;
-    alpha[p] = -expm1f(-expf(row[0]));
+    const auto feat = [&](int f) { return kDirect ? ldf(h + (int64_t)F * p + f) : rows[lane * kHeadStride + f]; };
+    alpha[p] = -expm1f(-expf(feat(0)));
     float c[4];
 #pragma unroll
     for (int ch = 0; ch < 4; ++ch) {
       float s = 0.f;
 #pragma unroll
-      for (int q = 0; q < 9; ++q) s = fmaf(Y[q], row[1 + 9 * ch + q], s);
+      for (int q = 0; q < 9; ++q) s = fmaf(Y[q], feat(1 + 9 * ch + q), s);
       c[ch] = s;
     }
     reinterpret_cast<float4*>(color)[p] = make_float4(c[0], c[1], c[2], c[3]);
@@ -242,15 +258,19 @@ extern "C" inpc_status inpc_sh_head_fwd(const inpc_camera* cam, const float* pos
   if (!alpha_out || !color_out || !aligned(color_out, 16)) return fail(INPC_ERR_INVALID_ARG, "bad output pointer");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const ShConsts k = make_consts(*cam);
-  // rows of 40 or more features whose 4-element groups are aligned
-  const bool vec = n_channels % 4 == 0 && n_channels >= 40 && aligned(h, h_dtype == INPC_F32 ? 16 : 8);
+  const bool four = aligned(h, h_dtype == INPC_F32 ? 16 : 8);
+  const Rows how = n_channels % 4 ? Rows::kDirect : four && n_channels >= 40 ? Rows::kVec : Rows::kOne;
   const auto run = [&](auto kernel, auto* rows) {
     kernel<<<grid_for_warps(n), kHeadThreads, 0, s>>>(k, pos, rows, n, n_channels, alpha_out, color_out);
   };
-  const float* hf = static_cast<const float*>(h);
-  const __nv_bfloat16* hb = static_cast<const __nv_bfloat16*>(h);
-  if (h_dtype == INPC_F32) vec ? run(k_sh_head_fwd<float, true>, hf) : run(k_sh_head_fwd<float, false>, hf);
-  else vec ? run(k_sh_head_fwd<__nv_bfloat16, true>, hb) : run(k_sh_head_fwd<__nv_bfloat16, false>, hb);
+  const auto read = [&](auto* rows) {
+    using HT = std::remove_const_t<std::remove_pointer_t<decltype(rows)>>;
+    if (how == Rows::kVec) run(k_sh_head_fwd<HT, Rows::kVec>, rows);
+    else if (how == Rows::kOne) run(k_sh_head_fwd<HT, Rows::kOne>, rows);
+    else run(k_sh_head_fwd<HT, Rows::kDirect>, rows);
+  };
+  if (h_dtype == INPC_F32) read(static_cast<const float*>(h));
+  else read(static_cast<const __nv_bfloat16*>(h));
   return check_launch("k_sh_head_fwd");
 }
 
