@@ -27,14 +27,63 @@ namespace {
 // (the memory of the backward's pairs).
 __device__ __forceinline__ float* splat_values(const RasterWs& ws) { return reinterpret_cast<float*>(ws.fscal); }
 
-// A warp per pixel, over pixels that lie a grid of warps apart (neighbouring
-// ones, whose points they share, are walked at the same time).  One lane each
-// reads the buckets of the warp's next 32 pixels, so empty pixels cost no
-// chain of loads, and a pixel's order entries are read while the one before is
-// walked.  1M points at 640 x 416: 37.8 -> 33.5 us, near the L2's rate of
-// partly written sectors (4.2M stores, 125G/s); 100,000 points at 1200 x 800
-// 66 -> 43 us.  32 consecutive pixels per warp instead: 64 and 40 us.
-constexpr int kSplatCtas = 8;  // per SM
+// The pixels with at most 8 blended fragments (`few`: the lanes that hold their
+// bucket start, size, count and place), four at a time on 8 lanes each, the next
+// four's order read while these are walked.  The product scan of 8 lanes is the
+// one of 32 on its first 8, so the values are the same bits.
+__device__ __forceinline__ void few_splat_weights(const RP& P, const RasterWs& ws, float* __restrict__ val,
+                                                  unsigned few, uint32_t s0, int m, int nb, int qx, int qy) {
+  const Group<8> L;
+  const int g = L.base_lane >> 3;
+  int j = 0, jnb = 0;
+  uint32_t js0 = 0;
+  uint2 o = make_uint2(0, 0);
+  const auto next = [&]() {  // this group's next pixel and its order entries
+    unsigned f = few;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (i < g) f &= f - 1;
+    const bool any = f != 0;
+    j = any ? __ffs(f) - 1 : 0;
+    jnb = __shfl_sync(0xffffffffu, nb, j);
+    js0 = __shfl_sync(0xffffffffu, s0, j);
+    const int jm = __shfl_sync(0xffffffffu, m, j);
+    if (!any) jnb = 0;
+    if (L.lg < jnb) o = order_at(P, ws, js0, jm, L.lg);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) few &= few - 1;  // 0 stays 0
+  };
+  bool more = few != 0;
+  if (more) next();
+  while (more) {
+    const int cnb = jnb, cx = __shfl_sync(0xffffffffu, qx, j), cy = __shfl_sync(0xffffffffu, qy, j);
+    const uint32_t cs0 = js0;
+    const uint2 co = o;
+    more = few != 0;
+    if (more) next();
+    const bool valid = L.lg < cnb;
+    float a = 0.f;
+    uint32_t dst = 0;
+    if (valid) {
+      a = ws.alpha[cs0 + co.x];
+      dst = frag_index(ws, co.y, cx, cy);
+    }
+    const ChunkT<8> ct = chunk_transmittance<8>(L, P, a, valid, cnb, 1.0f);
+    if (L.lg < ct.take) val[dst] = __fmul_rn(ct.Tk, a);
+  }
+}
+
+// Pixels that lie a grid of warps apart (neighbouring ones, whose points they
+// share, are walked at the same time), 32 to a warp: one lane each reads their
+// buckets, so empty pixels cost no chain of loads; pixels of up to 8 blended
+// fragments go four at a time, the others a warp each, a pixel's order entries
+// read while the one before is walked.  A warp for every pixel leaves most of
+// its lanes idle and most of its time in one pixel's chain of loads: 300,000
+// points at 1280 x 832 141 -> 56 us (a grid-stride loop over all pixels 103),
+// 600,000 at 1920 x 1080 256 -> 90, 4M there (8 fragments a pixel) 395 -> 224;
+// 1M leaf-grouped points at 640 x 416 the same, near the L2's rate of partly
+// written sectors (4.2M stores, 125G/s).  The times are of the whole call.
+constexpr int kSplatCtas = 8;  // per SM (5, 6 and 7: 4M points 252, 233 us; leaf-grouped ones 73, 68 and 67, with 8 66)
 __global__ void __launch_bounds__(256, kSplatCtas) k_pixel_splat_weights(RP P, const int32_t* __restrict__ n_contrib,
                                                                         RasterWs ws) {
   const Group<32> G;
@@ -50,7 +99,9 @@ __global__ void __launch_bounds__(256, kSplatCtas) k_pixel_splat_weights(RP P, c
       m = (int)(ws.pix_start[mine + 1] - s0);
       nb = blended_count(n_contrib, mine, m);
     }
-    unsigned todo = __ballot_sync(0xffffffffu, nb > 0);
+    const int qy = (int)((uint32_t)mine / (uint32_t)P.cam.W), qx = (int)((uint32_t)mine - (uint32_t)qy * P.cam.W);
+    few_splat_weights(P, ws, val, __ballot_sync(0xffffffffu, nb > 0 && nb <= 8), s0, m, nb, qx, qy);
+    unsigned todo = __ballot_sync(0xffffffffu, nb > 8);
     uint2 o_next = make_uint2(0, 0);
     const auto first_order = [&]() {  // of the next pixel
       if (!todo) return;
@@ -63,8 +114,7 @@ __global__ void __launch_bounds__(256, kSplatCtas) k_pixel_splat_weights(RP P, c
     while (todo) {
       const int j = __ffs(todo) - 1;
       todo &= todo - 1;
-      const long long q = w0 + j * n_warps;
-      const int qy = (int)(q / P.cam.W), qx = (int)(q - (long long)qy * P.cam.W);
+      const int jqx = G.bcast(qx, j), jqy = G.bcast(qy, j);
       const uint32_t js0 = G.bcast(s0, j);
       const int jm = G.bcast(m, j), jnb = G.bcast(nb, j);
       uint2 o = o_next;
@@ -76,7 +126,7 @@ __global__ void __launch_bounds__(256, kSplatCtas) k_pixel_splat_weights(RP P, c
         uint32_t dst = 0;
         if (valid) {
           a = ws.alpha[js0 + o.x];
-          dst = frag_index(ws, o.y, qx, qy);
+          dst = frag_index(ws, o.y, jqx, jqy);
         }
         const ChunkT<32> ct = chunk_transmittance<32>(G, P, a, valid, min(32, jnb - b), T);
         if (G.lg < ct.take) val[dst] = __fmul_rn(ct.Tk, a);
