@@ -277,12 +277,19 @@ __global__ void __launch_bounds__(kClassThreads) k_classify(long long n_pix, Cla
 // bucket): the tile kernel takes nb <= cap.small, a lane group per pixel (the
 // back of the list) nb <= cap.large, a warp per pixel (its front) nb <=
 // kCandMax, the CTA path the rest.
+// kThree: the three classes occur (lane groups below a warp).
+template <bool kThree>
 __global__ void k_classify_bwd(const int32_t* __restrict__ n_contrib, long long n_pix, ClassCaps cap, RasterWs ws) {
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   uint32_t nb = 0;
   if (q < n_pix) {
     const int c = n_contrib[q];
     nb = c < 0 ? 0u : min((uint32_t)c, ws.pix_start[q + 1] - ws.pix_start[q]);
+  }
+  if constexpr (!kThree) {
+    if (nb > (uint32_t)kCandMax) ws.heavy[atomicAdd(ws.heavy_count, 1u)] = (uint32_t)q;
+    else if (nb > cap.small) ws.large[n_pix - 1 - atomicAdd(ws.wide_count, 1u)] = (uint32_t)q;
+    return;
   }
   // one lane per class goes to its counter, the classes' round trips together
   const int cls = nb <= cap.small ? 0 : nb <= cap.large ? 1 : nb <= (uint32_t)kCandMax ? 2 : 3;
@@ -2400,7 +2407,7 @@ inpc_status launch_blend_bwd(const RP& P, const FT* feat, const int32_t* n_contr
   INPC_CUDA(cudaMemsetAsync(ws.heavy_count, 0, 6 * sizeof(uint32_t), s), "clear class counts");
   const ClassCaps cap{2 * GA, 4 * GA, bwd_group_cap<GA>()};
   INPC_TIMED("k_classify_bwd", s,
-             k_classify_bwd<<<(unsigned)ceil_div(P.n_pix, 256), 256, 0, s>>>(n_contrib, P.n_pix, cap, ws));
+             k_classify_bwd<(GA < 32)><<<(unsigned)ceil_div(P.n_pix, 256), 256, 0, s>>>(n_contrib, P.n_pix, cap, ws));
   INPC_TRY(check_launch("k_classify_bwd"));
   // together or one by one, as in the forward
   const unsigned sm = (unsigned)device_sm_count();
