@@ -2380,16 +2380,22 @@ inpc_status launch_fwd(const RP& P, const float* pos, const float* opacity, cons
   // (32 views of 1M samples over 8 streams 37.9-39.6 ms, the lists first
   // 40.0-40.4).
   // The CTA path waits for all (it takes over what the warps leave open).
+  // Whole-warp widths need the warps' launch for selections only, of which
+  // there are kSelectMin or none: with too few fragments for that it is left
+  // out (64 views of 262,144 samples at 320 x 240 over 8 streams 20.4 -> 20.3 ms, behind the
+  // persistent front end 18.2 -> 17.9).
+  const bool may_select = P.n_pix >= kSelectMin && 4 * P.n >= (long long)kSelectMin * (kCandMax + 1);
+  const bool with_warps = GA < 32 || may_select;
   if (P.together) {
-    INPC_TRY(warps(0));
-    INPC_TRY(wide(1));
+    if (with_warps) INPC_TRY(warps(0));
+    INPC_TRY(wide(with_warps));
     INPC_TRY(mid(1));
     INPC_TRY(tiles(1));
   } else {
     INPC_TRY(tiles(0));
     INPC_TRY(mid(0));
     INPC_TRY(wide(0));
-    INPC_TRY(warps(0));
+    if (with_warps) INPC_TRY(warps(0));
   }
   INPC_TIMED("k_blend_fwd_heavy", s,
              k_blend_fwd_heavy<V, GA, FT><<<device_sm_count() * 4, kThreads, HeavyBuf::bytes(), s>>>(
