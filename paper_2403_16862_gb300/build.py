@@ -35,8 +35,8 @@ def _sources():
 
 def _stamp(srcs) -> str:
     h = hashlib.sha256()
-    for f in srcs + [os.path.join(CSRC, x) for x in sorted(os.listdir(CSRC)) if x.endswith(".cuh")] + \
-            [os.path.join(ROOT, "include", "inpc.h")]:
+    for f in srcs + [os.path.join(d, x) for d in (CSRC, os.path.join(ROOT, "include")) for x in sorted(os.listdir(d))
+                     if x.endswith((".cuh", ".h"))]:
         with open(f, "rb") as fh:
             h.update(f.encode() + fh.read())
     h.update(" ".join(ARCH + FLAGS).encode())
