@@ -93,27 +93,41 @@ KERNELS = ["k_draw_count", "k_place", "k_hash_fwd", "k_pix_count", "k_pix_scatte
 # reported as null rather than as figures of another kernel.
 CAPTURED = {"k_point_grad_hash": {"traffic": 696_609_792 + 218_087_680, "l2_reductions": 243_198_353,
                                   "stamp": "5cfcc33073ce2e3f"}}
-# the sources each kernel's code comes from (stamped for CAPTURED); "step":
-# every kernel of one view
-KERNEL_SOURCES = {"k_point_grad_hash": ["raster_bwd.cu", "raster_impl.cuh", "hashgrid_impl.cuh", "common.cuh"],
-                  "k_hash_fwd": ["hashgrid.cu", "hashgrid_impl.cuh", "common.cuh"],
-                  "step": ["sample.cu", "sample_impl.cuh", "scan.cuh", "hashgrid.cu", "hashgrid_impl.cuh",
-                           "raster_impl.cuh", "raster_fwd.cu", "raster_bwd.cu", "common.cuh"]}
+# the translation units each kernel's code comes from; stamped (for CAPTURED)
+# with everything they include.  "step": every kernel of one view
+KERNEL_SOURCES = {"k_point_grad_hash": ["raster_bwd.cu"],
+                  "k_hash_fwd": ["hashgrid.cu"],
+                  "step": ["sample.cu", "hashgrid.cu", "raster_fwd.cu", "raster_fwd_wide.cu", "raster_bwd.cu"]}
 # DRAM bytes (read + write) of every kernel of one view on the full workload,
 # the library's kernels and the table-gradient clear, summed from one ncu
 # capture of all launches (mean of its 5 views); profiles/ holds the command
 STEP_CAPTURED = {"dram_bytes": 7_219_000_000, "stamp": "fbcef1a1402290b5"}
 
 
+def source_files(units):
+    """The translation units and the files they include, in a fixed order."""
+    import re
+    todo = [os.path.join(ROOT, "paper_2403_16862_gb300", "csrc", u) for u in units]
+    found = set(todo)
+    while todo:
+        f = todo.pop()
+        with open(f) as fh:
+            names = re.findall(r'^\s*#include\s+"([^"]+)"', fh.read(), flags=re.M)
+        new = {os.path.normpath(os.path.join(os.path.dirname(f), n)) for n in names} - found
+        found |= new
+        todo += new
+    return sorted(found)
+
+
 def source_stamp(kernel):
     import hashlib
-    files = KERNEL_SOURCES.get(kernel)
-    if not files:
+    units = KERNEL_SOURCES.get(kernel)
+    if not units:
         return None
     h = hashlib.sha256()
-    for f in files:
-        with open(os.path.join(ROOT, "paper_2403_16862_gb300", "csrc", f), "rb") as fh:
-            h.update(f.encode() + fh.read())
+    for f in source_files(units):
+        with open(f, "rb") as fh:
+            h.update(os.path.basename(f).encode() + fh.read())
     return h.hexdigest()[:16]
 
 
