@@ -27,8 +27,9 @@ def _ptr(t):
 
 
 def _stream():
-    # torch.cuda.current_stream().cuda_stream without the Stream object (3.2 us a call)
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    # the handle without the Stream object (3.2 us a call) where torch offers it
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
 
 
 def _need(t, dtype, name, device=None):
