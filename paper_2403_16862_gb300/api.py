@@ -422,7 +422,8 @@ def multisample_render(tree_t, root_size: float, desc, table, cam, seed: int, n_
                        opts=None, lambda_l: float = 0.5, max_rounds: int = 8):
     """Inference multisampling (Sec. 3.2): k view-specific point clouds (view
     ids 0..k-1 of this seed), each queried and rasterized, their feature
-    images averaged per pixel.  Returns the FP32 average image."""
+    images averaged per pixel.  Returns the FP32 average image.  Up to four
+    images are held at a time, as many as fit 2 GiB (one always)."""
     c, l, p = tree_t
     opts = opts or RasterOptions(n_channels=desc.n_levels * desc.n_feats, head_mode=True)
     w = view_weights(c, l, p, root_size, cam, lambda_l=lambda_l)
