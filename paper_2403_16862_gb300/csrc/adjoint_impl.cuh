@@ -27,8 +27,8 @@ inline bool grad_levels_fit_l2(const GridParams& P, int l_first) {
 // reductions (x and x + 1 with the same y, z: rows differing in their low
 // bits) usually fall in one 128-byte line and cost one L1 wavefront.
 //
-// fine(): the lane's four corner contributions straight to L2.
-// coarse(): the lane keeps one float4 accumulator per y-z corner in shared
+// add() of a fine lane: its four corner contributions straight to L2.
+// add() of a coarse lane keeps one float4 accumulator per y-z corner in shared
 // memory (acc[s kStride]) and sends a corner's sum to memory only when the
 // next point needs a different vertex in that slot.  The slot of vertex
 // (X, Y, Z) is given by the parities of X, Y and Z: every cell has exactly

@@ -3,8 +3,9 @@
 // leaf layout) and the per-point blending weights it consumes (App. A.6).
 //
 // Blending weights: after a forward, every pixel's blended prefix (recorded
-// by the forward in blending order) is walked once more with the forward's
-// own product scan, so T_k alpha_k is bitwise the forward's; each splat's
+// by the forward in blending order) is walked once more with the product scan
+// of whole warps: T_k alpha_k is bitwise the forward's for widths that whole
+// warps blend, and agrees to FP32 rounding for narrower ones; each splat's
 // value lands at its point's entry for the footprint corner it came from
 // and a per-point pass combines a point's four splats with their bilinear
 // weights.

@@ -20,14 +20,18 @@
 // Blending.  The scatter pass stores each fragment's alpha (Eq. 6 with the
 // clamp) beside its key, so blending gathers nothing but the feature rows of
 // the blended fragments.  T_k = prod_{j<k} (1 - alpha_j) is a product scan
-// across lanes (chunks of GA fragments on the group path, 256 on the CTA
-// path), the stopping fragment (first with T_{k+1} < t_min) comes from a
+// across lanes (chunks of GA fragments on the group path, of 32 within blocks
+// of 256 on the warp and CTA paths), the stopping fragment (first with T_{k+1} < t_min) comes from a
 // ballot, and sum_k T_k alpha_k c_k is an independent gather-reduce over the
 // feature rows (V channels per lane, float4 loads).
 //
-// Backward.  Per pixel, T_k is recomputed by the forward's own scan (same
-// rounding, nothing stored between the passes) and the suffix sums
-// S_k = sum_{j>k} T_j alpha_j (c_j . g) run back to front.  Each fragment's
+// Backward.  Per pixel, T_k is recomputed by a scan over the blended prefix
+// that the forward recorded (no transmittance is stored between the passes) and
+// the suffix sums S_k = sum_{j>k} T_j alpha_j (c_j . g) run back to front.
+// Widths of whole warps (GA = 32) scan as the forward did, to the same bits; for
+// narrower ones a pixel may change paths (a bucket that the forward blended by
+// warps and of which a few fragments count, or the other way round), and its T_k
+// agree to FP32 rounding.  Each fragment's
 // two scalars (T_k alpha_k, dL/dalpha_k) go to the point's entry for the
 // footprint corner the fragment came from (point-major, zero where nothing
 // blended); a per-point kernel then reads its four pairs together, gathers
@@ -2006,8 +2010,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_fwd_heavy(RP P, const FT*
   }
 }
 
-// Backward of the pixels with more than kRegMax * GA blended fragments: the
-// whole CTA on one pixel, over the blended prefix the forward recorded (no
+// Backward of the pixels with more than kCandMax blended fragments: the whole
+// CTA on one pixel, over the blended prefix the forward recorded (no
 // sort); T_k and c_k . g in shared memory (or, beyond kHeavyKeys, in the
 // global scratch kb).
 struct HeavyBwdBuf {

@@ -271,8 +271,11 @@ __device__ bool cube_outside(const Cam& cam, const double c[3], double e) {
 // The same decision from FP32 where it is certain: 1 outside, 0 not, -1 too
 // close to a plane.  A plane's function is linear, so its extreme corner is
 // the center's value plus or minus the half edge times the absolute sum of
-// the coefficients; values within 2^-18 of the terms' magnitudes (16 times
-// what the dozen FP32 roundings can add up to) are left to cube_outside.
+// the coefficients; values within 2^-18 of the terms' magnitudes are left to
+// cube_outside.  (No term passes through more than 14 roundings of 2^-24 each
+// on its way into a value -- the products and sums of xc or of the
+// coefficients, the half edge, the last sum -- and 2^-18 is 64 of them, more
+// than four times as much.)
 // The eight corners take about 500 FP64 operations per leaf, which the FP64
 // pipe (a few lanes per SM and clock) turned into 140 us for 262,144 leaves.
 __device__ __forceinline__ int cube_outside_fp32(const Cam& cam, const float c[3], float half) {
