@@ -261,7 +261,10 @@ __device__ __forceinline__ bool blend_selected(const Group<32>& G, const RP& P, 
                                                long long q, WarpCand& S, const FT* __restrict__ feat,
                                                FT* __restrict__ image, float* __restrict__ T_final,
                                                int32_t* __restrict__ n_contrib) {
-  // 99 % of the benchmark scene's pixels blend at most 66 fragments
+  // A pixel that blends more than it selects is done again by a CTA.  2.5M points
+  // on 160 x 120 pixels (520 fragments each), 4 channels, forward with and
+  // without the selection: alphas of 0.2 to 0.8 (64 blended) 233 and 466 us; of
+  // 0.02 to 0.3 (220 blended) 1209 and 1159; of 0.001 to 0.01 (all) 1266 and 1216.
   constexpr int kLeast = 72, kMost = 128;
   uint32_t d[32];
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
