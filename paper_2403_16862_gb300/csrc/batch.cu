@@ -38,7 +38,8 @@ struct Events {
 // time cost more than they hide: 64 views of 262,144 samples at 320 x 240 over
 // 8 streams 21.8 ms together and 20.4 ms one by one, over 4 streams 19.7 and
 // 19.4.  With the persistent front end (rasterizer passes only) together is
-// better: 18.2 and 18.4 ms, 16 of those views 4.69 and 4.85 ms.
+// better for few views: 16 of those 4.65 and 4.79 ms, 8 views of 50,000 samples
+// 0.99 and 1.03; 64 of those over 8 streams 18.2 and 17.9.
 inpc_status run_raster(const inpc_hashgrid_desc* grid, const inpc_view_job& v, float* grad_table, inpc_stream_t s,
                        bool together) {
   INPC_TRY(rasterize_fwd(&v.cam, &v.opts, v.pos, nullptr, v.h, v.n_samples, v.image, v.T_final, v.n_contrib,
